@@ -12,32 +12,36 @@
 // 65504).  tcgen05.mma kind::f16 takes both operands in fp16 and accumulates
 // in fp32 in tensor memory.
 //
-// Structure (one CTA per 128-row x BN-token output tile, 18 warps; the
-// row tiles may belong to up to four matrices that share X, one launch for
-// a fused q/k/v or gate/up projection):
-//   warp 0     TMA producer for the fp16 activation tile (128B swizzle) and
-//              owner of the tensor-memory allocation;
-//   warp 1     a single elected thread issues tcgen05.mma (M=128, N=BN,
-//              K=16 per instruction, 4 per 64-wide k-block) with the weight
-//              operand A in tensor memory and the activations B in shared
-//              memory, and commits to the stage's "empty" barrier;
-//   warps 2-17 dequantise in two sets of eight that fill alternate stages:
+// Structure: persistent CTAs of 18 warps, one per SM, take output tiles of
+// 128 weight rows x BN = 64, 128 or 256 tokens in turn (the row tiles may
+// belong to up to four matrices that share X, one launch for a fused q/k/v or
+// gate/up projection).  A step is two 64-wide k-blocks (128 codes of a row):
+//   warp 0     TMA producer: fp16 activation tiles (128B swizzle), packed
+//              code tiles of 256 codes; owner of the tensor-memory allocation;
+//   warp 1     issues tcgen05.mma (M=128, N=BN, K=16 per instruction, 8 per
+//              step) with the weight operand A in tensor memory and the
+//              activations B in shared memory, and commits to the step's
+//              "empty" barrier;
+//   warps 2-17 dequantise in four groups of four that take every fourth step:
 //              each thread owns one weight row of the tile (its tensor-memory
-//              lane) and one 32-code half of its set's 64-wide k-blocks,
-//              loads those codes and their scale, forms fp16 s*c in natural
-//              k order and writes it to the stage's A columns of tensor
-//              memory with one tcgen05.st (shared memory then carries only
-//              the activation tiles: the MMA's operand reads, the TMA writes
-//              and no generic-proxy stores)
+//              lane), reads the step's 128 codes of it from shared memory and
+//              their scales from global memory, forms fp16 s*c in the k order
+//              of X's columns and writes it to the step's A columns of tensor
+//              memory (tcgen05.st; shared memory then carries no
+//              generic-proxy stores)
 //              (a group whose scale lets s*c reach 65520, checked per scale
 //              as |s| 2^(q-1) or |s| (2^q - 1) + |m|, raises SSS_FLAG_RANGE);
-//              after the last k-block the same warps drain the fp32
-//              accumulator with tcgen05.ld (each set of four warps one
-//              quarter of the columns) and store Y (for a fixed token, a warp writes
-//              32 consecutive floats).
-// Tensor memory (512 columns): the fp32 accumulator in columns [0, BN), the
-// A stages in columns BN + 32 s (one 64-wide fp16 k-block of 128 rows per
-// 32 columns: lane = row, two k-consecutive halves per 32-bit column).
+//              after a tile's last step the same warps drain its fp32
+//              accumulator with tcgen05.ld and store Y (for a fixed token, a
+//              warp writes 32 consecutive floats).
+// Tensor memory (512 columns): the fp32 accumulator (two for BN <= 128), then
+// four A stages of 64 columns (lane = row, two k-consecutive halves per 32-bit
+// column).
+// What bounds it: at BN = 256 the MMAs (1025 cycles a step; 512 per k-block is
+// the pipe's rate), 86 % of cuBLAS's burst rate at 2048 tokens with the
+// conversion of X (14336 x 4096 q = 4: 145 us; 192 us when a tile's k-blocks
+// each brought their own narrow code and scale tiles); at BN <= 128 the
+// dequantisation (590-730 cycles a step); at few tokens the launch itself.
 // Every mbarrier wait is bounded (about one second of global time); on
 // expiry the CTA raises SSS_FLAG_TIMEOUT, all roles leave their loops, and
 // the tensor memory is still released.
@@ -48,18 +52,14 @@
 #include <algorithm>
 #include <mutex>
 
-#include "sss_internal.cuh"
+#include "act_q8.cuh"
 
 namespace sss {
 namespace {
 
 constexpr int kBM = 128;            // weight rows per tile (MMA M)
 constexpr int kBK = 64;             // k per stage (128 bytes of fp16)
-constexpr int kDqWarps = 8;         // warps that fill one stage
-// threads of a CTA with SETS sets of 8 dequantising warps (on alternate
-// k-blocks), the producer warp and the MMA issuer's warp
-template <int SETS>
-constexpr int threads_of() { return 64 + 32 * kDqWarps * SETS; }
+constexpr int kThreads = 64 + 32 * 16;  // producer, MMA issuer, 16 dequantising warps
 constexpr uint64_t kWaitNs = 1000000000ull;  // bounded waits: 1 s
 
 // ---------------------------------------------------------------------------
@@ -96,6 +96,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// whether the phase has completed, without waiting
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait on a phase parity.  Returns false when the wait gave up,
 // either on its own time limit or because another role raised *abort.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
@@ -112,6 +124,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
       }
     }
   }
+}
+
+// One lane of the (converged) warp.  The producer and issuer loops run warp-wide
+// and elect a lane only around the instruction itself: their counters,
+// addresses and descriptors then stay in uniform registers.  Run by one lane
+// under divergent control flow, each tcgen05 instruction first moves its
+// operands there (45 cycles apiece unloaded, about 200 beside the busy
+// dequantising warps), and a k-block's issue took longer than its MMAs.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(p));
+  return p != 0;
 }
 
 __device__ __forceinline__ void tc_fence_before() {
@@ -201,71 +227,120 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 // ---------------------------------------------------------------------------
-// Dequantisation of 32 codes of one row into 16 natural-order fp16 pairs.
+// Dequantisation of 32 codes of one row into 16 fp16 pairs.
+//
+// Pair p holds the two elements whose fields a single shift brings to bit 0
+// of the two 16-bit halves of a code word: q = 4: elements 8w + i and
+// 8w + i + 4 (p = 4w + i); q = 2, 3: elements 16w + e and 16w + e + 8
+// (p = 8w + e).  The k order inside a k-block is free as long as both
+// operands use it, so the conversion of X stores its columns in this order
+// (x16_kernel) and no byte permutes are needed here: a shift and one LOP3
+// per pair, against a mask, a PRMT and an OR in natural order.
 // ---------------------------------------------------------------------------
 
-// PRMT selector: result = [a.byte_i, 0, b.byte_i, 0]; the zero bytes use the
-// sign-replicate mode on a byte whose top bit is clear.
-__device__ __forceinline__ uint32_t pair_bytes(uint32_t a, uint32_t b, int i) {
-  const uint32_t sel = static_cast<uint32_t>(i) | (static_cast<uint32_t>(8 + i) << 4) |
-                       (static_cast<uint32_t>(4 + i) << 8) |
-                       (static_cast<uint32_t>(12 + i) << 12);
-  uint32_t r;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
-  return r;
-}
-
-// u pairs (natural order: element 2p in the low half, 2p+1 in the high half)
-// of a 32-code sub-chunk, as 16-bit integers.
+// Words of sub-chunk i (32 codes) of a thread's 128 codes: lo[] (q = 4: 4
+// words, else 2) and for q = 3 its high-bit plane word hi.
 template <int Q>
-__device__ __forceinline__ void code_pairs(const uint32_t* w, uint32_t (&u)[16]) {
-  if constexpr (Q == 4) {
+struct Codes128 {
+  static constexpr int NW = Q == 4 ? 16 : 8;
+  uint32_t lo[NW];
+  uint32_t hi[Q == 3 ? 4 : 1];
+};
+
+// w: the 4q words of 128 consecutive codes as they lie in memory; q = 3
+// keeps its planes per group of G codes.
+template <int Q>
+__device__ __forceinline__ void order_codes(const uint32_t (&w)[4 * Q], int G, Codes128<Q>& c) {
+  if constexpr (Q == 3) {
+    if (G == 32) {
 #pragma unroll
-    for (int wi = 0; wi < 4; ++wi) {
-      const uint32_t ev = w[wi] & 0x0F0F0F0Fu, od = (w[wi] >> 4) & 0x0F0F0F0Fu;
+      for (int i = 0; i < 4; ++i) {
+        c.lo[2 * i] = w[3 * i];
+        c.lo[2 * i + 1] = w[3 * i + 1];
+        c.hi[i] = w[3 * i + 2];
+      }
+    } else if (G == 64) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) u[4 * wi + i] = pair_bytes(ev, od, i);
+      for (int i = 0; i < 4; ++i) {
+        const int b = 6 * (i >> 1), h = i & 1;
+        c.lo[2 * i] = w[b + 2 * h];
+        c.lo[2 * i + 1] = w[b + 2 * h + 1];
+        c.hi[i] = w[b + 4 + h];
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) c.lo[i] = w[i];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) c.hi[i] = w[8 + i];
     }
   } else {
 #pragma unroll
-    for (int wi = 0; wi < 2; ++wi) {
-      const uint32_t a = w[wi] & 0x03030303u, b = (w[wi] >> 2) & 0x03030303u;
-      const uint32_t c = (w[wi] >> 4) & 0x03030303u, d = (w[wi] >> 6) & 0x03030303u;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        u[8 * wi + 2 * i] = pair_bytes(a, b, i);
-        u[8 * wi + 2 * i + 1] = pair_bytes(c, d, i);
-      }
-    }
-    if constexpr (Q == 3) {
-      const uint32_t hi = w[2];
-#pragma unroll
-      for (int p = 0; p < 16; ++p) {
-        const uint32_t v = (hi >> (2 * p)) & 3u;
-        u[p] |= ((v & 1u) << 2) | ((v & 2u) << 17);  // + 4*hi bit, both halves
-      }
-    }
+    for (int i = 0; i < 4 * Q; ++i) c.lo[i] = w[i];
   }
 }
 
-template <int Q>
-__device__ __forceinline__ void load_sub32(const uint8_t* __restrict__ row, int64_t grp, int sc,
-                                           int G, bool valid, uint32_t* w) {
-  if constexpr (Q == 4) {
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (valid) v = __ldcs(reinterpret_cast<const uint4*>(row + grp * (G / 2) + sc * 16));
-    w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-  } else if constexpr (Q == 2) {
-    uint2 v = make_uint2(0, 0);
-    if (valid) v = __ldcs(reinterpret_cast<const uint2*>(row + grp * (G / 4) + sc * 8));
-    w[0] = v.x; w[1] = v.y;
-  } else {
-    w[0] = w[1] = w[2] = 0;
-    if (valid) {
-      const uint32_t* base = reinterpret_cast<const uint32_t*>(row + grp * (3 * G / 8));
-      w[0] = __ldcs(base + 2 * sc);
-      w[1] = __ldcs(base + 2 * sc + 1);
-      w[2] = __ldcs(base + G / 16 + sc);
+// (a & b) | c in one LOP3
+__device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+// fp16 2^(10 - pos) in both halves, for pos = 0, step, 2 step, ... (step 4 for
+// q = 4, else 2)
+constexpr int kMagics = 5;
+
+// the high-plane bits of elements 16w .. 16w + 15 (w = half of the plane
+// word) spread to every other bit: element 16w + e at bit 2e (e < 8) and
+// element 16w + 8 + e at bit 16 + 2e
+__device__ __forceinline__ uint32_t spread_high(uint32_t plane, int w) {
+  uint32_t x = __byte_perm(plane, 0u, w ? 0x4342u : 0x4140u);
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  x = (x | (x << 1)) & 0x55555555u;
+  return x;
+}
+
+// The fp16 pairs of sub-chunk i: RN16(s c), or RN16(s u + m) for ASYM.  A
+// field u at bit pos of a half, OR-ed into the mantissa of 2^(10 - pos), is
+// the fp16 value 2^(10 - pos) + u: it needs no shift of its own while it
+// ends below bit 10 (q = 4: pos 0, 4; q = 2: 0 .. 8; q = 3: 0 .. 6 with its
+// high bit), so one shift per word serves half of its fields.
+// The magic words come in registers (mg, from kernel arguments): as literals
+// the compiler splits the mask and the OR, or moves the literal into a
+// register each time (208 ALU instructions per 128 codes, 2 issue cycles
+// each, against 64 LOP3 and 16 shifts).
+template <int Q, bool ASYM>
+__device__ __forceinline__ void dequant32(const Codes128<Q>& c, int i, __half2 s2, __half2 m2,
+                                          const uint32_t (&mg)[kMagics],
+                                          uint32_t (&out)[16]) {
+  constexpr int PW = Q == 4 ? 4 : 8;                   // pairs per word
+  constexpr int DIRECT = Q == 4 ? 2 : (Q == 2 ? 5 : 4);  // fields taken before the shift
+  constexpr int BITS = Q == 4 ? 4 : 2;                 // distance of the fields
+#pragma unroll
+  for (int w = 0; w < 16 / PW; ++w) {
+    const uint32_t v0 = c.lo[i * (16 / PW) + w], v1 = v0 >> (DIRECT * BITS);
+    uint32_t h0 = 0u, h1 = 0u;
+    if constexpr (Q == 3) {
+      const uint32_t hs = spread_high(c.hi[i], w);
+      h0 = hs << 2;
+      h1 = hs >> (DIRECT * BITS - 2);
+    }
+#pragma unroll
+    for (int e = 0; e < PW; ++e) {
+      const int pos = BITS * (e < DIRECT ? e : e - DIRECT);
+      const uint32_t field = ((1u << BITS) - 1u) << pos;
+      uint32_t mag = and_or(e < DIRECT ? v0 : v1, field | (field << 16), mg[pos / BITS]);
+      if constexpr (Q == 3) {
+        const uint32_t hb = 4u << pos;
+        mag = and_or(e < DIRECT ? h0 : h1, hb | (hb << 16), mag);
+      }
+      // minus 2^(10 - pos) (+ 2^(q-1) for symmetric codes): exact
+      __half2 hv = *reinterpret_cast<const __half2*>(&mag);
+      const __half2 bias =
+          __float2half2_rn(static_cast<float>((1 << (10 - pos)) + (ASYM ? 0 : 1 << (Q - 1))));
+      hv = __hsub2(hv, bias);                             // c (or u) exactly
+      hv = ASYM ? __hfma2(hv, s2, m2) : __hmul2(hv, s2);  // RN16(s*c) / RN16(s*u+m)
+      out[PW * w + e] = *reinterpret_cast<const uint32_t*>(&hv);
     }
   }
 }
@@ -279,7 +354,7 @@ struct GemmJob {
   const uint16_t* mins;
   float* y;  // [m][n]
   int64_t n;
-  int64_t tile0;
+  int tile0;
 };
 struct GemmArgs {
   GemmJob job[kMaxGemmJobs];
@@ -287,90 +362,252 @@ struct GemmArgs {
   uint32_t* status;
   int64_t m, k;
   int G;
+  uint32_t magic[kMagics];  // dequant32's magic words
+  int vec;    // the scales (and mins) of 128 codes can be loaded as one vector
   int stall;  // test hook: the first stage's weight tile is never announced
   // split K: CTA z of nsplit takes k-blocks [z * chunk, ...) and leaves its
   // fp32 tile in part + z * m * np (row tile t at rows 128 t .. 128 t + 127
   // of np = 128 x all row tiles); the last of a tile's splits to finish
   // (counted in cnt, zero on entry) sums them in split order into y
   int nsplit;
+  int chunk;  // k-blocks per split, a multiple of kWK
+  int rt, mt, items;  // row tiles, token tiles, rt x mt x nsplit
   int64_t np;
   float* part;
   int* cnt;
 };
 
-// The activation tile map, and per matrix its code and scale tile maps
-// (used with TW).
+// The activation tile map, and per matrix its code tile map (used with CT).
 struct GemmMaps {
   CUtensorMap x;
   CUtensorMap c[kMaxGemmJobs];
-  CUtensorMap s[kMaxGemmJobs];
 };
 
-// Shared memory: STAGES activation tiles (1024-aligned for the 128-byte
-// swizzle), then with TW the stages' packed-code tiles (128 rows x 8q bytes)
-// and scale windows (128 rows x 8 fp16), then the barriers.
-template <int BN, int STAGES, int Q, bool TW>
+// A thread owns one weight row and takes 128 codes (two k-blocks) of it at a
+// time; a code tile is 128 rows x 256 codes (kWK k-blocks, 32q bytes a row).
+// Code tiles this wide matter: the TMA unit moves about one box row per 1.7
+// cycles whatever the row's length, so a tile per k-block (32-byte rows, and
+// as many 16-byte rows of scales) cost as much as the activation tile and
+// set the pace: 640 cycles per k-block at 128 tokens with nothing else to do.
+constexpr int kWK = 4;      // k-blocks per code tile
+constexpr int kAStages = 4; // A operand steps (two k-blocks) in tensor memory
+// A barrier tells a wait for one phase from the next by its parity alone, so
+// whoever waits on one has to wait for every phase in turn.  The dequantising
+// groups take every fourth step and every other code tile: the A stages are a
+// multiple of four and the code tiles an even number, which gives each group
+// stages of its own.
+
+// Shared memory: XS activation tiles (1024-aligned for the 128-byte
+// swizzle), then with CT the code tiles, then the barriers.
+template <int BN, int Q, bool CT>
 struct Smem {
-  static constexpr int B_BYTES = BN * kBK * 2;               // 16 or 32 KB
-  static constexpr int C_BYTES = TW ? kBM * 8 * Q : 0;       // codes of one k-block
-  static constexpr int S_BYTES = TW ? kBM * 16 : 0;          // 8 scales per row
-  static constexpr int STAGE = B_BYTES;
-  static constexpr int C_OFF = STAGES * B_BYTES;
-  static constexpr int S_OFF = C_OFF + STAGES * C_BYTES;
-  static constexpr int BAR_OFF = S_OFF + STAGES * S_BYTES;
-  static constexpr int TOTAL = BAR_OFF + (3 * STAGES + 1) * 8 + 16 + 1024;  // + align slack
-  static constexpr int A_COL = BN;                // first A-stage column in tensor memory
+  static constexpr int XS = BN == 256 ? 3 : 4;               // activation stages (steps)
+  static constexpr int WS = BN == 256 ? 2 : 4;               // code tiles in flight
+  static constexpr int X_BYTES = BN * kBK * 2;               // one k-block: 8, 16 or 32 KB
+  static constexpr int W_BYTES = CT ? kBM * 32 * Q : 0;
+  static constexpr int W_OFF = XS * 2 * X_BYTES;
+  static constexpr int BAR_OFF = W_OFF + WS * W_BYTES;
+  static constexpr int NB = BN == 256 ? 1 : 2;               // accumulators
+  static constexpr int NBAR = XS + 2 * kAStages + 2 * WS + 2 * NB + 1;
+  static constexpr int TOTAL = BAR_OFF + NBAR * 8 + 16 + 1024;  // + align slack
+  static constexpr int A_COL = NB * BN;           // first A-stage column in tensor memory
+  static_assert(kAStages % 4 == 0 && WS % 2 == 0 && XS <= kAStages, "see kAStages");
   static_assert(TOTAL <= 227 * 1024, "shared memory per CTA");
+  static_assert(NB * BN + 64 * kAStages <= 512, "tensor memory holds accumulators and A stages");
 };
-// tensor-memory columns a CTA allocates: all 512 with one CTA per SM, half
-// when two CTAs (one dequantising set each) share an SM
-template <int SETS>
-constexpr int tmem_cols_of() { return SETS == 1 ? 256 : 512; }
+constexpr int kTmemCols = 512;  // one CTA per SM
 
-// TW: the packed codes and scales arrive by TMA with the activation tile
-// (q = 2, 4 on the symmetric grids, where a k-block's codes are 16-byte
-// aligned); otherwise each dequantising thread loads its own from global
-// memory a few k-blocks ahead.
-template <int Q, bool ASYM, int BN, int STAGES, bool TW, int SETS>
-__global__ void __launch_bounds__(threads_of<SETS>(), SETS == 1 ? 2 : 1)
+// The 4q words of codes of tile row `row`, half `h` (128 codes) of a code
+// tile in shared memory.  The tile is stored with the swizzle of its row
+// length (q = 4: 128 bytes, chunk ^ (row & 7); q = 2: 64 bytes, chunk ^
+// ((row >> 1) & 3)), so a quarter-warp's 16-byte loads fall in distinct
+// banks; the 96-byte rows of q = 3 are unswizzled (two-way conflicts).
+template <int Q>
+__device__ __forceinline__ void load_tile_codes(uint32_t tile, int row, int h,
+                                                uint32_t (&w)[4 * Q]) {
+  const uint32_t base = tile + static_cast<uint32_t>(row * 32 * Q);
+  const uint32_t sw = Q == 4 ? (row & 7) : (Q == 2 ? ((row >> 1) & 3) : 0);
+#pragma unroll
+  for (int c = 0; c < Q; ++c) {
+    const uint32_t a = base + 16u * (static_cast<uint32_t>(Q * h + c) ^ sw);
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(w[4 * c]), "=r"(w[4 * c + 1]), "=r"(w[4 * c + 2]), "=r"(w[4 * c + 3])
+                 : "r"(a));
+  }
+}
+
+// The fp16 scales (or mins) of the four 32-code sub-chunks of 128 codes
+// whose first group is gi, as u16 pairs; groups past the row's nG read as 0.
+__device__ __forceinline__ uint2 load_scales(const uint16_t* __restrict__ row, int64_t gi,
+                                             int64_t nG, int G, bool vec) {
+  if (G == 32) {
+    if (vec) return __ldg(reinterpret_cast<const uint2*>(row + gi));
+    uint32_t v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = gi + i < nG ? __ldg(row + gi + i) : 0u;
+    return make_uint2(v[0] | (v[1] << 16), v[2] | (v[3] << 16));
+  }
+  uint32_t a, b;
+  if (G == 64) {
+    if (vec) {
+      const uint32_t v = __ldg(reinterpret_cast<const uint32_t*>(row + gi));
+      a = v & 0xFFFFu;
+      b = v >> 16;
+    } else {
+      a = __ldg(row + gi);
+      b = gi + 1 < nG ? __ldg(row + gi + 1) : 0u;
+    }
+  } else {
+    a = b = __ldg(row + gi);
+  }
+  return make_uint2(a | (a << 16), b | (b << 16));
+}
+__device__ __forceinline__ uint16_t scale_of(const uint2& v, int i) {
+  const uint32_t w = (i & 2) ? v.y : v.x;
+  return static_cast<uint16_t>((i & 1) ? (w >> 16) : (w & 0xFFFFu));
+}
+
+// What an output tile (and K split) of the launch's item list is: items run
+// over the row tiles of all matrices first, then token tiles, then splits.
+struct Item {
+  int jb;               // matrix
+  int tx, ty, z;        // row tile (of all matrices), token tile, split
+  int n0, m0;           // first row (in its matrix) and token
+  int kb_base, nkb;     // its k-blocks: kb_base + kb for kb = 0 .. nkb - 1
+  int nsteps;           // of two k-blocks (the last may hold one)
+};
+__device__ __forceinline__ Item item_of(const GemmArgs& a, int it, int BN) {
+  Item w;
+  w.tx = it % a.rt;
+  const int rest = it / a.rt;
+  w.ty = rest % a.mt;
+  w.z = rest / a.mt;
+  w.jb = 0;
+  while (w.jb + 1 < a.njobs && w.tx >= a.job[w.jb + 1].tile0) ++w.jb;
+  w.n0 = (w.tx - a.job[w.jb].tile0) * kBM;
+  w.m0 = w.ty * BN;
+  w.kb_base = w.z * a.chunk;
+  w.nkb = min(static_cast<int>(a.k / kBK) - w.kb_base, a.chunk);
+  w.nsteps = (w.nkb + 1) / 2;
+  return w;
+}
+
+// The end of a K split's item, by the 512 dequantising threads: the tile's last
+// split to arrive sums the partials in split order (z = 0, 1, ...: the same
+// order whichever split is last) into y and leaves the counter at zero.
+// Returns false, to every thread, when some thread's ok is false.
+__device__ __forceinline__ bool sum_splits(const GemmArgs& a, const Item& e, int BN, bool ok,
+                                        volatile int* last) {
+  __threadfence();  // this CTA's partial tile, device-wide
+  uint32_t bad;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred p, 1, 512, q;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(bad)
+      : "r"(ok ? 0u : 1u)
+      : "memory");
+  if (bad) return false;
+  int* cnt = a.cnt + e.ty * a.rt + e.tx;
+  if (threadIdx.x == 64) *last = atomicAdd(cnt, 1) == a.nsplit - 1;
+  asm volatile("bar.sync 1, 512;" ::: "memory");
+  if (!*last) return true;
+  __threadfence();
+  // 4 consecutive rows per element (n % 4 == 0, y and the partials 16-byte
+  // aligned); four elements per thread at a time, so their loads of a split
+  // are in flight together
+  const GemmJob& job = a.job[e.jb];
+  constexpr int kV = kBM / 4;  // float4 per token of the tile
+  constexpr int kE = 4;
+  const int64_t mn = a.m * a.np;
+  const int64_t g0 = static_cast<int64_t>(e.tx) * kBM;
+#pragma unroll 1
+  for (int e0 = threadIdx.x - 64; e0 < kV * BN; e0 += kE * 512) {
+    float4 acc[kE];
+    int64_t off[kE];
+    bool in[kE];
+#pragma unroll
+    for (int j = 0; j < kE; ++j) {
+      const int el = e0 + j * 512;
+      const int64_t mm = e.m0 + el / kV, rr = static_cast<int64_t>(e.n0) + 4 * (el % kV);
+      in[j] = el < kV * BN && mm < a.m && rr < job.n;
+      off[j] = in[j] ? mm * a.np + g0 + 4 * (el % kV) : 0;
+      acc[j] = in[j] ? __ldcg(reinterpret_cast<const float4*>(a.part + off[j]))
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int z = 1; z < a.nsplit; ++z) {
+      float4 v[kE];
+#pragma unroll
+      for (int j = 0; j < kE; ++j)
+        v[j] = in[j] ? __ldcg(reinterpret_cast<const float4*>(a.part + z * mn + off[j]))
+                     : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < kE; ++j) {
+        acc[j].x += v[j].x; acc[j].y += v[j].y; acc[j].z += v[j].z; acc[j].w += v[j].w;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kE; ++j) {
+      const int el = e0 + j * 512;
+      if (in[j])
+        *reinterpret_cast<float4*>(job.y + static_cast<int64_t>(e.m0 + el / kV) * job.n + e.n0 +
+                                   4 * (el % kV)) = acc[j];
+    }
+  }
+  if (threadIdx.x == 64) *cnt = 0;
+  return true;
+}
+
+// Persistent: one CTA per SM takes items blockIdx.x, + gridDim.x, ...  The
+// steps of all its items are numbered through, each item starting at an even
+// number, so that step P uses A stage P % 4, is dequantised by group P % 4 and
+// lies in code tile P / 2.  While an item's last MMAs run and its accumulator
+// is drained, the next item's tiles load and its first steps dequantise; with
+// up to 128 tokens per tile there are two accumulators, and the next item's
+// MMAs run through the drain as well.  (One CTA per item spent about 9000 of
+// 27000 cycles at 128 tokens and k = 4096 on its start and end.)
+//
+// CT: the packed codes arrive by TMA (rows of k q / 8 bytes, a multiple of
+// 16); otherwise (q = 3 with k an odd multiple of 64) each dequantising
+// thread loads its own from global memory one step ahead.
+template <int Q, bool ASYM, int BN, bool CT>
+__global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmArgs a) {
-  using S = Smem<BN, STAGES, Q, TW>;
-  constexpr int kTmemCols = tmem_cols_of<SETS>();
-  static_assert(BN + 32 * STAGES <= kTmemCols, "tensor memory holds the accumulator and A stages");
+  using S = Smem<BN, Q, CT>;
+  constexpr int XS = S::XS, WS = S::WS, NB = S::NB;
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment for the swizzle atoms
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint64_t* full_a = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);
-  uint64_t* full_b = full_a + STAGES;
-  uint64_t* empty = full_b + STAGES;
-  uint64_t* done = empty + STAGES;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  uint64_t* full_x = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);
+  uint64_t* full_w = full_x + XS;
+  uint64_t* empty_w = full_w + WS;
+  uint64_t* full_a = empty_w + WS;
+  uint64_t* empty = full_a + kAStages;  // of both operands of a step
+  uint64_t* done = empty + kAStages;    // an item's MMAs have completed
+  uint64_t* acc_free = done + NB;       // its accumulator has been read
+  uint64_t* retired = acc_free + NB;    // used when a wait has run out
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(retired + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* last = abort + 1;
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  // this CTA's matrix jb, its rows n0 .. n0 + 127 in that matrix, and the
-  // same rows g0 .. g0 + 127 of the partial tiles
-  int jb = 0;
-  while (jb + 1 < a.njobs && static_cast<int64_t>(blockIdx.x) >= a.job[jb + 1].tile0) ++jb;
-  const GemmJob& job = a.job[jb];
-  const int64_t n0 = (static_cast<int64_t>(blockIdx.x) - job.tile0) * kBM;
-  const int64_t g0 = static_cast<int64_t>(blockIdx.x) * kBM;
-  const int64_t m0 = static_cast<int64_t>(blockIdx.y) * BN;
-  // this split's k-blocks: global k-block kb_base + kb for kb = 0 .. nkb - 1
-  const int nkb_all = static_cast<int>(a.k / kBK);
-  const int chunk = (nkb_all + a.nsplit - 1) / a.nsplit;
-  const int kb_base = static_cast<int>(blockIdx.z) * chunk;
-  const int nkb = min(nkb_all - kb_base, chunk);
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full_a[s], kDqWarps);
-      mbar_init(&full_b[s], 1);
+    for (int s = 0; s < XS; ++s) mbar_init(&full_x[s], 1);
+    for (int s = 0; s < kAStages; ++s) {
+      mbar_init(&full_a[s], 4);  // the four warps that cover the 128 rows
       mbar_init(&empty[s], 1);
     }
-    mbar_init(done, 1);
+    for (int s = 0; s < WS; ++s) {
+      mbar_init(&full_w[s], 1);
+      mbar_init(&empty_w[s], 8);  // the warps of its two 128-code halves
+    }
+    for (int s = 0; s < NB; ++s) {
+      mbar_init(&done[s], 1);
+      mbar_init(&acc_free[s], 16);
+    }
+    mbar_init(retired, 1);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -392,300 +629,417 @@ __global__ void __launch_bounds__(threads_of<SETS>(), SETS == 1 ? 2 : 1)
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   if (warp == 0) {
-    // ---------------- TMA producer: activation tiles ----------------
-    if (lane == 0) {
-      int issued = 0;
-      for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = static_cast<uint32_t>(kb / STAGES) & 1u;
-        if (!mbar_wait(&empty[s], ph ^ 1u, abort)) break;
-        unsigned char* sb = smem + s * S::STAGE;
-        mbar_arrive_expect_tx(&full_b[s], S::B_BYTES + S::C_BYTES + S::S_BYTES);
-        tma_load_2d(&maps.x, &full_b[s], sb, (kb_base + kb) * kBK, static_cast<int>(m0));
-        if constexpr (TW) {
-          // the k-block's codes (8q bytes of each row, x a multiple of 16) and
-          // the 8-scale window holding its groups (x rounded down to 8)
-          tma_load_2d(&maps.c[jb], &full_b[s], smem + S::C_OFF + s * S::C_BYTES,
-                      (kb_base + kb) * 8 * Q, static_cast<int>(n0));
-          tma_load_2d(&maps.s[jb], &full_b[s], smem + S::S_OFF + s * S::S_BYTES,
-                      ((kb_base + kb) * kBK / a.G) & ~7, static_cast<int>(n0));
-        }
-        issued = kb + 1;
-      }
-      if (*abort) {
-        // let this CTA's copies still in flight land before the CTA exits
-        int drain = 0;
-        for (int kb = std::max(0, issued - STAGES); kb < issued; ++kb)
-          (void)mbar_wait(&full_b[kb % STAGES], static_cast<uint32_t>(kb / STAGES) & 1u, &drain);
-      }
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc(kBM, BN);
-      // stage s: A at tensor-memory column A_COL + 32 s, B at shared offset
-      // s * STAGE (its descriptor's start-address field moves by STAGE / 16)
-      const uint32_t ta0 = tmem + static_cast<uint32_t>(S::A_COL);
-      const uint64_t bdesc0 = sw128_desc(smem_u32(smem));
-      constexpr uint64_t bstep = static_cast<uint64_t>(S::STAGE >> 4);
-      for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % STAGES;
-        const uint32_t ph = static_cast<uint32_t>(kb / STAGES) & 1u;
-        if (!mbar_wait(&full_a[s], ph, abort)) break;
-        if (!mbar_wait(&full_b[s], ph, abort)) break;
-        tc_fence_after();
-        umma_kblock(tmem, ta0 + static_cast<uint32_t>(32 * s), bdesc0 + bstep * s, idesc,
-                    kb == 0 ? 1u : 0u);
-        umma_commit(&empty[s]);  // frees the stage once these MMAs complete
-      }
-      umma_commit(done);
-    }
-  } else {
-    // ---------------- dequantise, then epilogue ----------------
-    // a warp may touch tensor-memory lanes 32*(warp % 4) .. +31 only, so
-    // thread (warp, lane) owns tile row 32*(warp % 4) + lane; the dequant
-    // warps w = warp - 2 form four groups of four (w >> 2), each covering
-    // the 128 rows once: group g takes the 32-code half hf = g & 1 of the
-    // k-blocks kb = set, set + SETS, ... of set g >> 1
-    const int row_i = 32 * (warp & 3) + lane;
-    const int hf = ((warp - 2) >> 2) & 1;
-    const int set = (warp - 2) >> 3;
-    bool big = false;  // a group whose s*c may leave the fp16 range
+    // ---------------- TMA producer: activation and code tiles ----------------
+    int sx = 0, xn = 0;      // activation stage, and how many steps were issued
+    int sw = 0, wn = 0;      // code stage, and how many tiles were issued
+    uint32_t phx = 0, phw = 0;
+    uint32_t used = 0;       // bit s: the parity of A stage s's next use
+    uint32_t hist = 0;       // the last steps' A stages and parities, 4 bits each
+    int P = 0;
     bool ok = true;
-    // fp16 s*c (ASYM: s*u + m) of the thread's 32 codes w into stage s's A
-    // columns 16 hf .. 16 hf + 15 of lane row_i, then the arrive
-    auto emit = [&](const uint32_t* w, uint16_t s16, uint16_t m16, int s, int kb) {
-      {
-        const __half sh = __ushort_as_half(s16);
-        const __half2 s2 = __halves2half2(sh, sh);
-        __half2 m2 = __float2half2_rn(0.f);
-        const float sa = fabsf(__half2float(sh));
-        if constexpr (!ASYM) big |= sa * static_cast<float>(1 << (Q - 1)) >= 65520.f;
-        if constexpr (ASYM) {
-          const __half mh = __ushort_as_half(m16);
-          m2 = __halves2half2(mh, mh);
-          big |= sa * static_cast<float>((1 << Q) - 1) + fabsf(__half2float(mh)) >= 65520.f;
+    for (int it = blockIdx.x; it < a.items && ok; it += gridDim.x) {
+      const Item w = item_of(a, it, BN);
+      const int nw = CT ? (w.nsteps + 1) / 2 : 0;
+      // code tile i of the item: 32q bytes (256 codes) of each row
+      auto put_w = [&](int i) -> bool {
+        const bool freed = mbar_wait(&empty_w[sw], phw ^ 1u, abort);
+        if (!__all_sync(0xffffffffu, freed)) return false;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(&full_w[sw], S::W_BYTES);
+          tma_load_2d(&maps.c[w.jb], &full_w[sw], smem + S::W_OFF + sw * S::W_BYTES,
+                      (w.kb_base + i * kWK) * 8 * Q, w.n0);
         }
-        uint32_t u[16];
-        code_pairs<Q>(w, u);
-        uint32_t out[16];
-#pragma unroll
-        for (int p = 0; p < 16; ++p) {
-          // 1024 + u as fp16, minus 1024 (+ 2^(q-1) for symmetric codes): exact
-          const uint32_t mag = u[p] | 0x64006400u;
-          __half2 hv = *reinterpret_cast<const __half2*>(&mag);
-          const __half2 bias = ASYM ? __float2half2_rn(1024.f)
-                                    : __float2half2_rn(static_cast<float>(1024 + (1 << (Q - 1))));
-          hv = __hsub2(hv, bias);                               // c (or u) exactly
-          hv = ASYM ? __hfma2(hv, s2, m2) : __hmul2(hv, s2);    // RN16(s*c) / RN16(s*u+m)
-          out[p] = *reinterpret_cast<const uint32_t*>(&hv);
+        __syncwarp();
+        if (++sw == WS) {
+          sw = 0;
+          phw ^= 1u;
         }
-        tmem_st16(tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) +
-                      static_cast<uint32_t>(S::A_COL + 32 * s + 16 * hf),
-                  out);
-      }
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      tc_fence_before();  // the stores, then the arrive the MMA issuer waits on
-      __syncwarp();
-      // (sss_test_set_stall: warp 2 leaves the first stage one arrive
-      // short, so the MMA issuer's wait for it runs out)
-      if (lane == 0 && !(a.stall && kb == 0 && warp == 2)) mbar_arrive(&full_a[s]);
-    };
-    if constexpr (TW) {
-      for (int kb = set; kb < nkb; kb += SETS) {
-        const int s = kb % STAGES;
-        const uint32_t ph = static_cast<uint32_t>(kb / STAGES) & 1u;
-        // warp-uniform, since the tensor-memory stores are .sync.aligned:
-        // the stage's A columns are free and its code and scale tiles landed
-        const bool freed = mbar_wait(&empty[s], ph ^ 1u, abort);
-        if (!__all_sync(0xffffffffu, freed)) {
+        ++wn;
+        return true;
+      };
+      // code tiles run one ahead of the activations: their codes have the
+      // dequantisation before them
+      ok = nw == 0 || put_w(0);
+      for (int p = 0; p < w.nsteps && ok; ++p) {
+        if (p % 2 == 0 && p / 2 + 1 < nw && !put_w(p / 2 + 1)) {
           ok = false;
           break;
         }
-        const bool landed = mbar_wait(&full_b[s], ph, abort);
-        if (!__all_sync(0xffffffffu, landed)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();  // the MMAs that read this stage have completed
-        const unsigned char* cs = smem + S::C_OFF + s * S::C_BYTES + row_i * (8 * Q) + hf * (4 * Q);
-        uint32_t w[4] = {0u, 0u, 0u, 0u};
-        if constexpr (Q == 4) {
-          const uint4 v = *reinterpret_cast<const uint4*>(cs);
-          w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
-        } else {
-          const uint2 v = *reinterpret_cast<const uint2*>(cs);
-          w[0] = v.x; w[1] = v.y;
-        }
-        const int kg = kb_base + kb;
-        const int gi = (kg * kBK + 32 * hf) / a.G, g0 = (kg * kBK / a.G) & ~7;
-        const uint16_t s16 = *reinterpret_cast<const uint16_t*>(
-            smem + S::S_OFF + s * S::S_BYTES + row_i * 16 + 2 * (gi - g0));
-        emit(w, s16, 0, s, kb);
-      }
-    } else {
-      const int64_t r = n0 + row_i;
-      const bool rok = r < job.n;
-      const int64_t nG = a.k / a.G;
-      const uint8_t* rowp = job.codes + (rok ? r : 0) * (a.k * Q / 8);
-      // codes and scale (and min) of this thread's half of one k-block
-      struct KBlock {
-        uint32_t w[4];
-        uint16_t s, m;
-      };
-      auto fetch = [&](KBlock& d, int kb) {
-        if (kb >= nkb) return;
-        const int64_t kc = static_cast<int64_t>(kb_base + kb) * kBK + 32 * hf;
-        const int64_t grp = kc / a.G;
-        const int sc = static_cast<int>((kc % a.G) / 32);
-        load_sub32<Q>(rowp, grp, sc, a.G, rok, d.w);
-        d.s = rok ? __ldcs(job.scales + r * nG + grp) : static_cast<uint16_t>(0);
-        if constexpr (ASYM) d.m = rok ? __ldcs(job.mins + r * nG + grp) : static_cast<uint16_t>(0);
-      };
-      // the global loads run kPrefetch of this thread's k-blocks ahead of use
-      constexpr int kPrefetch = 4;
-      KBlock ring[kPrefetch];
-#pragma unroll
-      for (int q0 = 0; q0 < kPrefetch; ++q0) fetch(ring[q0], set + SETS * q0);
-      for (int kb0 = set; kb0 < nkb && ok; kb0 += SETS * kPrefetch) {
-#pragma unroll
-        for (int q0 = 0; q0 < kPrefetch; ++q0) {
-          const int kb = kb0 + SETS * q0;
-          if (kb >= nkb || !ok) break;
-          const int s = kb % STAGES;
-          const uint32_t ph = static_cast<uint32_t>(kb / STAGES) & 1u;
-          // warp-uniform, since the tensor-memory stores are .sync.aligned
-          const bool freed = mbar_wait(&empty[s], ph ^ 1u, abort);
+        // the stage is free once the MMAs of XS steps ago have completed
+        if (xn >= XS) {
+          const uint32_t h = hist >> (4 * (XS - 1));
+          const bool freed = mbar_wait(&empty[(h >> 1) & 3u], h & 1u, abort);
           if (!__all_sync(0xffffffffu, freed)) {
             ok = false;
             break;
           }
-          tc_fence_after();  // the MMAs that read this stage have completed
-          emit(ring[q0].w, ring[q0].s, ring[q0].m, s, kb);
-          fetch(ring[q0], kb + SETS * kPrefetch);
+        }
+        if (elect_one()) {
+          // (a box past the end of k reads zeros)
+          unsigned char* dst = smem + sx * 2 * S::X_BYTES;
+          mbar_arrive_expect_tx(&full_x[sx], 2 * S::X_BYTES);
+          tma_load_2d(&maps.x, &full_x[sx], dst, (w.kb_base + 2 * p) * kBK,
+                      w.m0);
+          tma_load_2d(&maps.x, &full_x[sx], dst + S::X_BYTES, (w.kb_base + 2 * p + 1) * kBK,
+                      w.m0);
+        }
+        __syncwarp();
+        const uint32_t sa = static_cast<uint32_t>(P + p) & 3u;
+        hist = (hist << 4) | (sa << 1) | ((used >> sa) & 1u);
+        used ^= 1u << sa;
+        if (++sx == XS) {
+          sx = 0;
+          phx ^= 1u;
+        }
+        ++xn;
+      }
+      P += (w.nsteps + 1) & ~1;
+    }
+    if (*abort) {
+      // let this CTA's copies still in flight land before the CTA exits
+      int drain = 0;
+      for (int i = max(0, xn - XS); i < xn; ++i)
+        (void)mbar_wait(&full_x[i % XS], static_cast<uint32_t>(i / XS) & 1u, &drain);
+      for (int i = max(0, wn - WS); i < wn; ++i)
+        (void)mbar_wait(&full_w[i % WS], static_cast<uint32_t>(i / WS) & 1u, &drain);
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    // The step loop is unrolled over the A stages, so that their barriers and
+    // columns are offsets of uniform registers (the reduction puts the
+    // tensor-memory base into one), and the next step's barriers are tried
+    // while this step's MMAs issue.
+    constexpr uint32_t idesc = make_idesc(kBM, BN);
+    const uint32_t tm = __reduce_or_sync(0xffffffffu, tmem);
+    const uint64_t bdesc0 = sw128_desc(smem_u32(smem));
+    constexpr uint64_t bstep = static_cast<uint64_t>(S::X_BYTES >> 4);
+    bool go = true;
+    int sx = 0, P = 0, n = 0;  // activation stage, first step and number of the item
+    uint32_t phx = 0, used = 0;
+    for (int it = blockIdx.x; it < a.items && go; it += gridDim.x, ++n) {
+      const Item w = item_of(a, it, BN);
+      const int buf = n % NB;
+      const uint32_t acc = tm + static_cast<uint32_t>(buf * BN);
+      // the accumulator's previous item has been drained
+      const bool fr = mbar_wait(&acc_free[buf], (static_cast<uint32_t>(n / NB) & 1u) ^ 1u, abort);
+      if (!__all_sync(0xffffffffu, fr)) break;
+      tc_fence_after();
+      bool there = false;
+      const int end = P + w.nsteps;
+      for (int P0 = P & ~3; P0 < end && go; P0 += kAStages) {
+#pragma unroll
+        for (int s = 0; s < kAStages; ++s) {
+          if (P0 + s < P || P0 + s >= end || !go) continue;
+          if (!there) {
+            bool t = mbar_wait(&full_a[s], (used >> s) & 1u, abort);
+            t = t && mbar_wait(&full_x[sx], phx, abort);
+            if (!__all_sync(0xffffffffu, t)) {
+              go = false;
+              continue;
+            }
+          }
+          used ^= 1u << s;
+          tc_fence_after();
+          const uint64_t bd = bdesc0 + 2 * bstep * sx;
+          if (++sx == XS) {
+            sx = 0;
+            phx ^= 1u;
+          }
+          constexpr int kNext[4] = {1, 2, 3, 0};
+          const bool next = mbar_test_wait(&full_a[kNext[s]], (used >> kNext[s]) & 1u) &&
+                            mbar_test_wait(&full_x[sx], phx);
+          if (elect_one()) {
+            const uint32_t ta = tm + static_cast<uint32_t>(S::A_COL + 64 * s);
+            umma_kblock(acc, ta, bd, idesc, P0 + s == P ? 1u : 0u);
+            if (2 * (P0 + s - P) + 1 < w.nkb) umma_kblock(acc, ta + 32, bd + bstep, idesc, 0u);
+            umma_commit(&empty[s]);  // frees both operands' stages once these MMAs complete
+          }
+          there = __all_sync(0xffffffffu, next);
         }
       }
+      if (elect_one()) umma_commit(&done[buf]);
+      __syncwarp();
+      P += (w.nsteps + 1) & ~1;
     }
-    if (__any_sync(0xffffffffu, big) && lane == 0 && a.status != nullptr)
-      atomicOr(a.status, SSS_FLAG_RANGE);
-    // ---------------- epilogue ----------------
-    // a warp may read tensor-memory lanes 32*(warp % 4) .. +31; the four
-    // sets of four warps take one quarter of the columns each
-    const bool fin = ok && mbar_wait(done, 0, abort);
-    if (__all_sync(0xffffffffu, fin)) {  // warp-uniform: tcgen05.ld is .sync.aligned
-      tc_fence_after();
-      const int sub = warp & 3;
-      const int row_local = sub * 32 + lane;
-      const int64_t rr = n0 + row_local;
-      constexpr int kCols = BN / (kDqWarps * SETS / 4);
-      const int cbeg = ((warp - 2) >> 2) * kCols;
-#pragma unroll 1
-      for (int c0 = cbeg; c0 < cbeg + kCols; c0 += 32) {
-        uint32_t v[32];
-        tmem_ld32(tmem + (static_cast<uint32_t>(sub * 32) << 16) + c0, v);
-        // one split: y; several: this split's partial tile
-        const bool split = a.nsplit > 1;
-        float* dst = split ? a.part + static_cast<int64_t>(blockIdx.z) * a.m * a.np + g0 + row_local
-                           : job.y + rr;
-        const int64_t ld = split ? a.np : job.n;
-        if (rr < job.n) {
+    if (*abort) {  // MMAs still in flight must retire before the CTA's memory goes
+      int drain = 0;
+      if (elect_one()) umma_commit(retired);
+      __syncwarp();
+      (void)mbar_wait(retired, 0u, &drain);
+    }
+  } else {
+    // ---------------- dequantise, and the epilogues ----------------
+    // a warp may touch tensor-memory lanes 32*(warp % 4) .. +31 only, so
+    // thread (warp, lane) owns tile row 32*(warp % 4) + lane; the dequant
+    // warps w = warp - 2 form four groups of four (w >> 2), each covering
+    // the 128 rows once: group g takes the 128-code steps P with P % 4 = g
+    const int quad = warp & 3;
+    const int row_i = 32 * quad + lane;
+    const int slot = (warp - 2) >> 2;
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(32 * quad) << 16);
+    const int lg = a.G == 32 ? 5 : (a.G == 64 ? 6 : 7);
+    const int64_t nG = a.k >> lg;
+    bool big = false;  // a group whose s*c may leave the fp16 range
+    __half2 smax = __float2half2_rn(0.f);  // symmetric grids: the largest |s| seen
+    bool ok = true;
+    uint32_t mg[kMagics];
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const int64_t mm = m0 + c0 + c;
-            if (mm < a.m) dst[mm * ld] = __uint_as_float(v[c]);
+    for (int i = 0; i < kMagics; ++i) mg[i] = a.magic[i];
+    uint32_t used = 0;  // parity of this group's A stage
+    // the item at hand and this thread's row of it
+    Item w = {};
+    int P = 0;           // the item's first step
+    const uint16_t *srow = nullptr, *mrow = nullptr;
+    bool rok = false;
+    uint2 sv_n = make_uint2(0u, 0u), mv_n = make_uint2(0u, 0u);
+    uint32_t wn[CT ? 1 : 4 * Q];
+    // the scales (and without CT the codes) of the item's step p, one of this
+    // group's steps ahead (codes: rows are 8-byte aligned; the last step may
+    // hold one k-block only)
+    auto fetch = [&](int p) {
+      if (p >= w.nsteps || !rok) return;
+      const int64_t gi = (static_cast<int64_t>(w.kb_base) * kBK + 128 * static_cast<int64_t>(p)) >> lg;
+      sv_n = load_scales(srow, gi, nG, a.G, a.vec != 0);
+      if constexpr (ASYM) mv_n = load_scales(mrow, gi, nG, a.G, a.vec != 0);
+      if constexpr (!CT) {
+        const uint8_t* src = a.job[w.jb].codes + (static_cast<int64_t>(w.n0) + row_i) * (a.k * Q / 8) +
+                             (static_cast<int64_t>(w.kb_base) + 2 * static_cast<int64_t>(p)) * (8 * Q);
+        const int words = 2 * p + 1 < w.nkb ? 4 * Q : 2 * Q;
+#pragma unroll
+        for (int i = 0; i < 2 * Q; ++i) {
+          const uint2 v = 2 * i < words ? __ldcs(reinterpret_cast<const uint2*>(src) + i)
+                                        : make_uint2(0u, 0u);
+          wn[2 * i] = v.x;
+          wn[2 * i + 1] = v.y;
+        }
+      }
+    };
+    auto start_item = [&](int it) {
+      w = item_of(a, it, BN);
+      const GemmJob& job = a.job[w.jb];
+      const int64_t r = static_cast<int64_t>(w.n0) + row_i;
+      rok = r < job.n;
+      srow = job.scales + (rok ? r : 0) * nG;
+      if constexpr (ASYM) mrow = job.mins + (rok ? r : 0) * nG;
+      if (!rok) {
+        sv_n = mv_n = make_uint2(0u, 0u);
+        if constexpr (!CT) {
+#pragma unroll
+          for (int i = 0; i < 4 * Q; ++i) wn[i] = 0u;
+        }
+      }
+      fetch((slot - P) & 3);
+    };
+    // dequantise the item's step p (p = nsteps, past the end of an item of an
+    // odd number of steps: only its half of the code tile is handed back)
+    auto do_step = [&](int p, bool first) {
+      const uint2 sv = sv_n, mv = mv_n;
+      Codes128<Q> codes;
+      {
+        uint32_t wv[4 * Q];
+        if constexpr (CT) {
+          const int t = (P + p) >> 1;  // code tile
+          const int ws = t % WS;
+          const bool landed = mbar_wait(&full_w[ws], static_cast<uint32_t>(t / WS) & 1u, abort);
+          if (!__all_sync(0xffffffffu, landed)) {
+            ok = false;
+            return;
+          }
+          load_tile_codes<Q>(smem_u32(smem) + S::W_OFF + ws * S::W_BYTES, row_i, p & 1, wv);
+          // the codes are in registers before the TMA may overwrite the tile
+          // (without the fence the loads can still be in flight at the arrive)
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&empty_w[ws]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4 * Q; ++i) wv[i] = wn[i];
+        }
+        order_codes<Q>(wv, a.G, codes);
+      }
+      if (p >= w.nsteps) return;
+      fetch(p + 4);
+      if constexpr (!ASYM)
+        smax = __hmax2(smax, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&sv.x)),
+                                     __habs2(*reinterpret_cast<const __half2*>(&sv.y))));
+      // (the second k-block of a tile's odd last step is not multiplied)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const __half sh = __ushort_as_half(scale_of(sv, i));
+        const __half2 s2 = __halves2half2(sh, sh);
+        __half2 m2 = __float2half2_rn(0.f);
+        if constexpr (ASYM) {
+          const __half mh = __ushort_as_half(scale_of(mv, i));
+          m2 = __halves2half2(mh, mh);
+          big |= fabsf(__half2float(sh)) * static_cast<float>((1 << Q) - 1) +
+                     fabsf(__half2float(mh)) >= 65520.f;
+        }
+        uint32_t out[16];
+        dequant32<Q, ASYM>(codes, i, s2, m2, mg, out);
+        if (i == 0) {
+          // warp-uniform, since the tensor-memory stores are .sync.aligned:
+          // the MMAs that read this stage have completed
+          const bool freed = mbar_wait(&empty[slot], used ^ 1u, abort);
+          if (!__all_sync(0xffffffffu, freed)) {
+            ok = false;
+            return;
+          }
+          used ^= 1u;
+          tc_fence_after();
+        }
+        tmem_st16(lane_base + static_cast<uint32_t>(S::A_COL + 64 * slot + 16 * i), out);
+      }
+      // the stores, then the arrive the MMA issuer waits on
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      tc_fence_before();
+      __syncwarp();
+      // (sss_test_set_stall: warp 2 leaves the first stage one arrive short,
+      // so the MMA issuer's wait for it runs out)
+      if (lane == 0 && !(a.stall && first && p == 0 && warp == 2)) mbar_arrive(&full_a[slot]);
+    };
+
+    int n = 0;
+    bool begun = false;  // the item's first step of this group is done
+    if (static_cast<int>(blockIdx.x) < a.items) start_item(blockIdx.x);
+    for (int it = blockIdx.x; it < a.items && ok; it += gridDim.x, ++n) {
+      const int pad = (w.nsteps + 1) & ~1;
+      for (int p = ((slot - P) & 3) + (begun ? 4 : 0); p < pad && ok; p += 4) do_step(p, n == 0);
+      begun = false;
+      if (ok && it + static_cast<int>(gridDim.x) < a.items) {
+        P += pad;
+        start_item(it + gridDim.x);
+        const int p = (slot - P) & 3;
+        if (p < ((w.nsteps + 1) & ~1)) {
+          do_step(p, false);
+          begun = true;
+        }
+      }
+      // ---- epilogue of item e = it: a warp may read tensor-memory lanes
+      // 32*(warp % 4) .. +31; the four groups take alternate sets of 32 columns
+      const int buf = n % NB;
+      const bool fin = ok && mbar_wait(&done[buf], static_cast<uint32_t>(n / NB) & 1u, abort);
+      ok = __all_sync(0xffffffffu, fin);  // warp-uniform: tcgen05.ld is .sync.aligned
+      const Item e = item_of(a, it, BN);
+      const bool split = a.nsplit > 1;
+      if (ok) {
+        tc_fence_after();
+        const GemmJob& job = a.job[e.jb];
+        // one split: y; several: this split's partial tile
+        const int64_t ld = split ? a.np : job.n;
+        float* dst = split ? a.part + e.z * a.m * a.np + static_cast<int64_t>(e.tx) * kBM + row_i
+                           : job.y + e.n0 + row_i;
+        dst += e.m0 * ld;
+        const int mleft = static_cast<int>(a.m - e.m0 < BN ? a.m - e.m0 : BN);
+        const bool erok = static_cast<int64_t>(e.n0) + row_i < job.n;
+        // everything read: the MMAs may overwrite the accumulator
+        auto release = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_free[buf]);
+        };
+        if (32 * slot >= BN) release();
+#pragma unroll 1
+        for (int c0 = 32 * slot; c0 < BN; c0 += 128) {
+          uint32_t v[32];
+          tmem_ld32(lane_base + static_cast<uint32_t>(buf * BN + c0), v);
+          if (c0 + 128 >= BN) release();
+          if (erok) {
+            float* d = dst + c0 * ld;
+#pragma unroll
+            for (int c = 0; c < 32; ++c) {
+              if (c0 + c < mleft) *d = __uint_as_float(v[c]);
+              d += ld;
+            }
           }
         }
       }
+      // (all 16 warps meet here for each item, so that one whose wait ran out
+      // leaves no other at the barriers of the sum)
+      if (split && !sum_splits(a, e, BN, ok, last)) ok = false;
     }
+    if constexpr (!ASYM)
+      big = __half2float(__hmax(__low2half(smax), __high2half(smax))) *
+                static_cast<float>(1 << (Q - 1)) >= 65520.f;
+    if (__any_sync(0xffffffffu, big) && lane == 0 && a.status != nullptr)
+      atomicOr(a.status, SSS_FLAG_RANGE);
   }
 
-  if (a.nsplit > 1) __threadfence();  // this CTA's partial tile, device-wide
   tc_fence_before();
   __syncthreads();
   if (*abort && threadIdx.x == 0 && a.status != nullptr) atomicOr(a.status, SSS_FLAG_TIMEOUT);
-  if (a.nsplit > 1 && !*abort) {
-    // the tile's last split to arrive sums the partials in split order
-    // (z = 0, 1, ...: the same order whichever split is last) into y and
-    // leaves the counter at zero
-    int* cnt = a.cnt + blockIdx.y * gridDim.x + blockIdx.x;
-    volatile int* last = abort + 1;
-    if (threadIdx.x == 0) *last = atomicAdd(cnt, 1) == a.nsplit - 1;
-    __syncthreads();
-    if (*last) {
-      __threadfence();
-      // 4 consecutive rows per element (n % 4 == 0, y and the partials
-      // 16-byte aligned); eight elements per thread at a time, so every
-      // split's eight loads are in flight together
-      constexpr int kV = kBM / 4;  // float4 per token of the tile
-      constexpr int kE = 8;
-      const int64_t mn = a.m * a.np;
-      for (int e0 = threadIdx.x; e0 < kV * BN; e0 += kE * blockDim.x) {
-        float4 acc[kE];
-        int64_t off[kE];
-        bool in[kE];
-#pragma unroll
-        for (int j = 0; j < kE; ++j) {
-          const int e = e0 + j * blockDim.x;
-          const int64_t mm = m0 + e / kV, rr = n0 + 4 * (e % kV);
-          in[j] = e < kV * BN && mm < a.m && rr < job.n;
-          off[j] = in[j] ? mm * a.np + g0 + 4 * (e % kV) : 0;
-          acc[j] = in[j] ? __ldcg(reinterpret_cast<const float4*>(a.part + off[j]))
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        for (int z = 1; z < a.nsplit; ++z) {
-          float4 v[kE];
-#pragma unroll
-          for (int j = 0; j < kE; ++j)
-            v[j] = in[j] ? __ldcg(reinterpret_cast<const float4*>(a.part + z * mn + off[j]))
-                         : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int j = 0; j < kE; ++j) {
-            acc[j].x += v[j].x; acc[j].y += v[j].y; acc[j].z += v[j].z; acc[j].w += v[j].w;
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < kE; ++j) {
-          const int e = e0 + j * blockDim.x;
-          if (in[j])
-            *reinterpret_cast<float4*>(job.y + (m0 + e / kV) * job.n + n0 + 4 * (e % kV)) = acc[j];
-        }
-      }
-      if (threadIdx.x == 0) *cnt = 0;
-    }
-  }
   if (warp == 0) {
     tc_fence_after();
-    if (*abort) {  // MMAs still in flight must retire before the TMEM is released
-      int drain = 0;
-      (void)mbar_wait(done, 0, &drain);
-    }
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(kTmemCols)
                  : "memory");
   }
 }
 
-// bf16 -> fp16 activation conversion (round to nearest even)
+// The fp16 activation operand: bf16 X rounded to fp16 (nearest even), or with
+// Q8 the Q8_0 values fl16(fl16(d) q) of its blocks of 32, its columns stored
+// in the k order of the dequantised weights (dequant32): of every PERM columns
+// (8 for q = 4, 16 for q = 2, 3), position 2i + h holds column i + h PERM/2.  A thread converts 16 columns, so two
+// lanes share a Q8_0 block.  The first threads also zero the GEMM's ncnt
+// split counters.  HBM- or launch-bound: 2 bytes read, 2 written per value.
+template <int PERM, bool Q8>
 __global__ void __launch_bounds__(256)
-    bf16_to_f16_kernel(const uint16_t* __restrict__ x, __half* __restrict__ y, int64_t nvec) {
+    x16_kernel(const uint16_t* __restrict__ x, __half* __restrict__ y, int64_t nvec,
+               int* __restrict__ cnt, int ncnt, uint32_t* __restrict__ status) {
   // programmatic dependent launch: start once the preceding kernel (which
   // may still read the fp16 buffer) has completed
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nvec;
-       i += stride) {
-    const uint4 v = __ldcs(reinterpret_cast<const uint4*>(x) + i);
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    uint32_t o[4];
+  const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  for (int64_t i = t0; i < ncnt; i += stride) cnt[i] = 0;
+  // block-uniform trip count: with Q8 every lane joins the shuffles
+  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < nvec; base += stride) {
+    const int64_t i = base + threadIdx.x;  // columns 16 i .. 16 i + 15 of the flat array
+    const bool valid = i < nvec;
+    uint32_t w[8];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float lo = __uint_as_float(w[e] << 16);
-      const float hi = __uint_as_float(w[e] & 0xFFFF0000u);
-      __half2 h = __floats2half2_rn(lo, hi);
-      o[e] = *reinterpret_cast<uint32_t*>(&h);
+    for (int c = 0; c < 2; ++c) {
+      const uint4 v = valid ? __ldcs(reinterpret_cast<const uint4*>(x) + 2 * i + c)
+                            : make_uint4(0u, 0u, 0u, 0u);
+      w[4 * c] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
     }
-    reinterpret_cast<uint4*>(y)[i] = make_uint4(o[0], o[1], o[2], o[3]);
+    float f[16];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      f[2 * e] = __uint_as_float(w[e] << 16);
+      f[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u);
+    }
+    if constexpr (Q8) {
+      float amax = 0.f;
+      unsigned bad = 0, flags = 0;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        amax = fmaxf(amax, fabsf(f[e]));
+        bad |= is_nonfinite(f[e]);
+      }
+      amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+      bad |= __shfl_xor_sync(0xffffffffu, bad, 1);
+      uint16_t d16;
+      const float d = q8_scale(amax, bad != 0, &d16, &flags);
+      const float df = __half2float(__ushort_as_half(d16));
+      const float rd = d != 0.f ? __frcp_rn(d) : 0.f;
+#pragma unroll
+      for (int e = 0; e < 16; ++e)
+        f[e] = d != 0.f ? df * static_cast<float>(q8_code(f[e], d, rd)) : 0.f;
+      if (valid && (threadIdx.x & 1) == 0 && flags != 0u && status != nullptr)
+        atomicOr(status, flags);
+    }
+    if (valid) {
+      uint32_t o[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int ea = PERM == 8 ? 8 * (j >> 2) + (j & 3) : j;
+        __half2 h = __floats2half2_rn(f[ea], f[ea + PERM / 2]);
+        o[j] = *reinterpret_cast<uint32_t*>(&h);
+      }
+      reinterpret_cast<uint4*>(y)[2 * i] = make_uint4(o[0], o[1], o[2], o[3]);
+      reinterpret_cast<uint4*>(y)[2 * i + 1] = make_uint4(o[4], o[5], o[6], o[7]);
+    }
   }
 }
 
@@ -702,9 +1056,9 @@ size_t x16_bytes(int64_t m, int64_t k) {
   return (mm * kk * 2 + 255) / 256 * 256;
 }
 
-// How a call runs: tile width, dequantising sets per CTA, K splits.
+// How a call runs: tile width, K splits, and k-blocks per split.
 struct GemmPlan {
-  int bn, sets, nsplit;
+  int bn, nsplit, chunk;
 };
 
 // Workspace layout: fp16 X, then (split K) the partial tiles (rows padded to
@@ -717,142 +1071,48 @@ size_t split_bytes(int64_t rt, int64_t m, const GemmPlan& p) {
   return round256(static_cast<size_t>(p.nsplit) * m * rt * kBM * 4) + round256(tiles * 4);
 }
 
-// Largest K split (>= 2 to count) that fills the idle SMs with `tiles`
-// tiles, keeps every split non-empty and at least `min_kb` k-blocks long,
-// and whose partial tiles fit in the workspace (ws bytes); 1 if none.
-int split_for(int64_t k, int64_t rt, int64_t m, size_t ws, int bn, int64_t tiles, int64_t min_kb) {
-  const int64_t sms = device_sm_count();
-  const int64_t nkb = k / kBK;
-  int split = static_cast<int>(std::min<int64_t>(sms / std::max<int64_t>(tiles, 1), nkb / min_kb));
-  if (split >= 2) {  // every split non-empty: as many as chunks of ceil(nkb / split)
-    const int64_t chunk = (nkb + split - 1) / split;
-    split = static_cast<int>((nkb + chunk - 1) / chunk);
-  }
-  for (; split >= 2; --split) {
-    const GemmPlan p{bn, 2, split};
-    if (x16_bytes(m, k) <= ws && x16_bytes(m, k) + split_bytes(rt, m, p) <= ws) return split;
-  }
-  return 1;
-}
-
-// 256-token tiles when they cover the SMs (each weight tile is then
-// dequantised for twice the tokens, and a k-block's MMAs take about as long
-// at N = 256 as at N = 128).  Otherwise, when each split keeps at least 64
-// k-blocks, 256-token tiles with K split over as many CTAs as fill the SMs;
-// else 256-token tiles unsplit when 128-token tiles would need a second
-// wave; else 128-token tiles, split (at least 8 k-blocks each) when they
-// leave SMs idle.  The tile's last split sums all partials alone, so a split pays
-// only with enough k-blocks behind it.  (Two half-size CTAs per SM, one
-// dequantising set each, measured slower than one full CTA: their rings are
-// half as deep.)  rt: the row tiles of all the call's matrices.
+// The plan of least estimated time, in SM cycles: each SM's share of the items,
+// an item at a time, plus the launch's start and end, and for K splits the last
+// arrival's sum of the partial tiles.  Per k-block 64- and 128-token tiles take
+// about 290 cycles (the dequantisation's rate) and 256-token tiles 512 (the
+// MMAs').  Splits end on code-tile boundaries and keep at least 8 k-blocks.
+// rt: the row tiles of all the call's matrices; ws: the bytes the partial tiles
+// must fit in.  K is split only to fill SMs that the tiles leave idle.
 GemmPlan plan_gemm(int64_t rt, int64_t k, int64_t m, size_t ws) {
   const int64_t sms = device_sm_count();
-  if (m > 128) {
-    const int64_t tiles = rt * ((m + 255) / 256);
-    if (tiles >= sms) return {256, 2, 1};
-    const int split = split_for(k, rt, m, ws, 256, tiles, 64);
-    if (split >= 2) return {256, 2, split};
-    // 128-token tiles would take a second wave (each CTA the whole k-range
-    // again) where 256-token tiles take one
-    if (rt * ((m + 127) / 128) > sms) return {256, 2, 1};
+  const int64_t nkb = k / kBK;
+  GemmPlan best{128, 1, static_cast<int>((nkb + kWK - 1) / kWK * kWK)};
+  int64_t best_cost = INT64_MAX;
+  for (int bn : {64, 128, 256}) {
+    if (bn > 64 && m <= bn / 2) break;
+    const int64_t per = bn == 256 ? 512 : 280 + bn / 8;
+    const int64_t tiles = rt * ((m + bn - 1) / bn);
+    for (int64_t split = 1; split <= 32; ++split) {
+      const int64_t chunk = ((nkb + split - 1) / split + kWK - 1) / kWK * kWK;
+      if (split > 1 &&
+          (chunk < 8 || (nkb + chunk - 1) / chunk != split || tiles * split > sms))
+        continue;
+      const GemmPlan p{bn, static_cast<int>(split), static_cast<int>(chunk)};
+      if (split > 1 &&
+          (x16_bytes(m, k) > ws || x16_bytes(m, k) + split_bytes(rt, m, p) > ws))
+        continue;
+      const int64_t rounds = (tiles * split + sms - 1) / sms;
+      const int64_t drain = bn == 256 ? 2500 : 600;
+      const int64_t sum = split > 1 ? 500 + split * m * rt * kBM * 4 / 1000 : 0;
+      const int64_t cost = rounds * (std::min(chunk, nkb) * per + drain) + 16 * bn + sum;
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = p;
+      }
+    }
   }
-  const int64_t tiles = rt * ((m + 127) / 128);
-  if (tiles >= sms) return {128, 2, 1};
-  return {128, 2, split_for(k, rt, m, ws, 128, tiles, 8)};
+  return best;
 }
 
 int64_t row_tiles(const sss_qtensor_t* const* ts, int count) {
   int64_t rt = 0;
   for (int j = 0; j < count; ++j) rt += (ts[j]->n + kBM - 1) / kBM;
   return rt;
-}
-
-template <int Q, bool ASYM, int BN, bool TW, int SETS>
-cudaError_t run_gemm(const sss_qtensor_t* const* ts, float* const* ys, int count,
-                     const __half* x16, int64_t m, uint32_t* status, cudaStream_t stream,
-                     int nsplit, unsigned char* ws_split) {
-  constexpr int STAGES = (BN == 256) ? (TW ? 5 : 6) : 8;
-  using S = Smem<BN, STAGES, Q, TW>;
-  const sss_qtensor_t& t0 = *ts[0];  // k, q, group and grid are those of every matrix
-  EncodeTiledFn enc = tensor_map_encoder();
-  if (enc == nullptr) return cudaErrorNotSupported;
-  GemmMaps maps;
-  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(t0.k), static_cast<cuuint64_t>(m)};
-  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(t0.k) * 2};
-  const cuuint32_t box[2] = {kBK, BN};
-  const cuuint32_t estr[2] = {1, 1};
-  CUresult cr = enc(&maps.x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(x16), dims,
-                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
-  GemmArgs a;
-  memset(&a, 0, sizeof a);
-  int64_t tile0 = 0;
-  for (int j = 0; j < count; ++j) {
-    const sss_qtensor_t& t = *ts[j];
-    maps.c[j] = maps.x;  // placeholders unless TW
-    maps.s[j] = maps.x;
-    if constexpr (TW) {
-      // packed codes [n][k q / 8] bytes: one k-block is 8q bytes of 128 rows;
-      // scales [n][k / G] fp16: a window of 8 (16 bytes) of 128 rows; rows
-      // past n read as zero
-      const cuuint64_t cd[2] = {static_cast<cuuint64_t>(t.k * Q / 8), static_cast<cuuint64_t>(t.n)};
-      const cuuint64_t cs[1] = {static_cast<cuuint64_t>(t.k * Q / 8)};
-      const cuuint32_t cb[2] = {static_cast<cuuint32_t>(8 * Q), kBM};
-      cr = enc(&maps.c[j], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, t.codes, cd, cs, cb, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
-      const int64_t ng = t.k / t.group;
-      const cuuint64_t sd[2] = {static_cast<cuuint64_t>(ng), static_cast<cuuint64_t>(t.n)};
-      const cuuint64_t ss[1] = {static_cast<cuuint64_t>(ng * 2)};
-      const cuuint32_t sbx[2] = {8, kBM};
-      cr = enc(&maps.s[j], CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, t.scales, sd, ss, sbx, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    }
-    a.job[j].codes = t.codes;
-    a.job[j].scales = t.scales;
-    a.job[j].mins = t.mins;
-    a.job[j].y = ys[j];
-    a.job[j].n = t.n;
-    a.job[j].tile0 = tile0;
-    tile0 += (t.n + kBM - 1) / kBM;
-  }
-  auto kern = gemm_kernel<Q, ASYM, BN, STAGES, TW, SETS>;
-  cudaError_t e = ensure_smem(kern, S::TOTAL);
-  if (e != cudaSuccess) return e;
-  a.njobs = count;
-  a.status = status;
-  a.m = m;
-  a.k = t0.k;
-  a.G = t0.group;
-  a.stall = (test_stall_mask() & SSS_TEST_STALL_GEMM) ? 1 : 0;
-  a.nsplit = nsplit;
-  a.np = tile0 * kBM;
-  a.part = nullptr;
-  a.cnt = nullptr;
-  const unsigned gx = static_cast<unsigned>(tile0);
-  const unsigned gy = static_cast<unsigned>((m + BN - 1) / BN);
-  if (nsplit > 1) {
-    a.part = reinterpret_cast<float*>(ws_split);
-    a.cnt = reinterpret_cast<int*>(ws_split + round256(static_cast<size_t>(nsplit) * m * a.np * 4));
-    e = cudaMemsetAsync(a.cnt, 0, sizeof(int) * gx * gy, stream);
-    if (e != cudaSuccess) return e;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(gx, gy, static_cast<unsigned>(nsplit));
-  cfg.blockDim = dim3(threads_of<SETS>(), 1, 1);
-  cfg.dynamicSmemBytes = S::TOTAL;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, maps, a);
 }
 
 struct GemmCall {
@@ -864,35 +1124,142 @@ struct GemmCall {
   uint32_t* status;
   cudaStream_t stream;
   GemmPlan plan;
-  unsigned char* ws_split;
+  float* part;
+  int* cnt;
 };
 
-template <int Q, bool ASYM, bool TW>
-cudaError_t gemm_tw(const GemmCall& c) {
-  if (c.plan.bn == 256)
-    return run_gemm<Q, ASYM, 256, TW, 2>(c.ts, c.ys, c.count, c.x16, c.m, c.status, c.stream,
-                                         c.plan.nsplit, c.ws_split);
-  return run_gemm<Q, ASYM, 128, TW, 2>(c.ts, c.ys, c.count, c.x16, c.m, c.status, c.stream,
-                                       c.plan.nsplit, c.ws_split);
+template <int Q, bool ASYM, int BN, bool CT>
+cudaError_t run_gemm(const GemmCall& c) {
+  using S = Smem<BN, Q, CT>;
+  const sss_qtensor_t& t0 = *c.ts[0];  // k, q, group and grid are those of every matrix
+  EncodeTiledFn enc = tensor_map_encoder();
+  if (enc == nullptr) return cudaErrorNotSupported;
+  GemmMaps maps;
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(t0.k), static_cast<cuuint64_t>(c.m)};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(t0.k) * 2};
+  const cuuint32_t box[2] = {kBK, BN};
+  const cuuint32_t estr[2] = {1, 1};
+  CUresult cr = enc(&maps.x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(c.x16), dims,
+                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  GemmArgs a;
+  memset(&a, 0, sizeof a);
+  const int64_t nG = t0.k / t0.group;
+  const int per = t0.group >= 128 ? 1 : 128 / t0.group;  // groups of 128 codes
+  bool vec = nG % per == 0;
+  int64_t tile0 = 0;
+  for (int j = 0; j < kMaxGemmJobs; ++j) {
+    maps.c[j] = maps.x;  // a placeholder where there is no code map
+    if (j >= c.count) continue;
+    const sss_qtensor_t& t = *c.ts[j];
+    if constexpr (CT) {
+      // packed codes [n][k q / 8] bytes: a tile is 32q bytes of 128 rows;
+      // bytes past the row and rows past n read as zero
+      const cuuint64_t cd[2] = {static_cast<cuuint64_t>(t.k * Q / 8), static_cast<cuuint64_t>(t.n)};
+      const cuuint64_t cs[1] = {static_cast<cuuint64_t>(t.k * Q / 8)};
+      const cuuint32_t cb[2] = {static_cast<cuuint32_t>(32 * Q), kBM};
+      cr = enc(&maps.c[j], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, t.codes, cd, cs, cb, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE,
+               Q == 4   ? CU_TENSOR_MAP_SWIZZLE_128B
+               : Q == 2 ? CU_TENSOR_MAP_SWIZZLE_64B
+                        : CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (cr != CUDA_SUCCESS) return cudaErrorInvalidValue;
+    }
+    vec = vec && reinterpret_cast<uintptr_t>(t.scales) % (2 * per) == 0 &&
+          (!ASYM || reinterpret_cast<uintptr_t>(t.mins) % (2 * per) == 0);
+    a.job[j].codes = t.codes;
+    a.job[j].scales = t.scales;
+    a.job[j].mins = t.mins;
+    a.job[j].y = c.ys[j];
+    a.job[j].n = t.n;
+    a.job[j].tile0 = tile0;
+    tile0 += (t.n + kBM - 1) / kBM;
+  }
+  auto kern = gemm_kernel<Q, ASYM, BN, CT>;
+  cudaError_t e = ensure_smem(kern, S::TOTAL);
+  if (e != cudaSuccess) return e;
+  a.njobs = c.count;
+  a.status = c.status;
+  a.m = c.m;
+  a.k = t0.k;
+  a.G = t0.group;
+  a.vec = vec ? 1 : 0;
+  for (int i = 0; i < kMagics; ++i) {
+    const int pos = (Q == 4 ? 4 : 2) * i;
+    const uint32_t h = pos <= 10 ? static_cast<uint32_t>(25 - pos) << 10 : 0u;
+    a.magic[i] = h | (h << 16);
+  }
+  a.stall = (test_stall_mask() & SSS_TEST_STALL_GEMM) ? 1 : 0;
+  a.nsplit = c.plan.nsplit;
+  a.chunk = c.plan.chunk;
+  a.np = tile0 * kBM;
+  a.part = c.part;
+  a.cnt = c.cnt;
+  const int64_t mt = (c.m + BN - 1) / BN;
+  const int64_t items = tile0 * mt * c.plan.nsplit;
+  if (items > INT32_MAX - 4096) return cudaErrorNotSupported;
+  a.rt = static_cast<int>(tile0);
+  a.mt = static_cast<int>(mt);
+  a.items = static_cast<int>(items);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(std::min<int64_t>(items, device_sm_count())), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = S::TOTAL;
+  cfg.stream = c.stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, maps, a);
+}
+
+template <int Q, bool ASYM, bool CT>
+cudaError_t gemm_bn(const GemmCall& c) {
+  switch (c.plan.bn) {
+    case 64: return run_gemm<Q, ASYM, 64, CT>(c);
+    case 128: return run_gemm<Q, ASYM, 128, CT>(c);
+    default: return run_gemm<Q, ASYM, 256, CT>(c);
+  }
 }
 
 template <int Q, bool ASYM>
-cudaError_t gemm_bn(const GemmCall& c) {
-  if constexpr (!ASYM && Q != 3) {
-    // the code and scale tiles by TMA: 16-byte aligned scale rows in every
-    // matrix
-    bool tw = ((c.ts[0]->k / c.ts[0]->group) * 2) % 16 == 0;
-    for (int j = 0; j < c.count; ++j)
-      tw = tw && (reinterpret_cast<uintptr_t>(c.ts[j]->scales) % 16) == 0;
-    if (tw) return gemm_tw<Q, ASYM, true>(c);
+cudaError_t gemm_ct(const GemmCall& c) {
+  // code rows a multiple of 16 bytes, as a tensor map needs (q = 2 and 4:
+  // always, since k % 64 == 0)
+  if constexpr (Q == 3) {
+    if (c.ts[0]->k % 128 != 0) return gemm_bn<Q, ASYM, false>(c);
   }
-  return gemm_tw<Q, ASYM, false>(c);
+  return gemm_bn<Q, ASYM, true>(c);
 }
 
 template <int Q>
 cudaError_t gemm_grid(const GemmCall& c) {
-  if (c.ts[0]->grid == SSS_GRID_ASYM) return gemm_bn<Q, true>(c);
-  return gemm_bn<Q, false>(c);
+  if (c.ts[0]->grid == SSS_GRID_ASYM) return gemm_ct<Q, true>(c);
+  return gemm_ct<Q, false>(c);
+}
+
+// X to the fp16 operand at x16, and the ncnt split counters at cnt to zero
+template <int PERM, bool Q8>
+cudaError_t run_x16(const uint16_t* x, __half* x16, int64_t m, int64_t k, int* cnt, int ncnt,
+                    uint32_t* status, cudaStream_t stream) {
+  const int64_t nvec = m * k / 16;
+  const int64_t want = (nvec + 255) / 256;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(std::max<int64_t>(
+                         1, std::min<int64_t>(want, static_cast<int64_t>(device_sm_count()) * 8))),
+                     1, 1);
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, x16_kernel<PERM, Q8>, x, x16, nvec, cnt, ncnt, status);
 }
 
 }  // namespace
@@ -916,31 +1283,29 @@ cudaError_t launch_gemm_multi(const sss_qtensor_t* const* ts, float* const* ys, 
                               uint32_t* status, cudaStream_t stream, bool act_q8) {
   if (count < 1 || count > kMaxGemmJobs) return cudaErrorInvalidValue;
   const int64_t k = ts[0]->k;
+  const int q = ts[0]->q;
   __half* x16 = static_cast<__half*>(workspace);
   const int64_t rt = row_tiles(ts, count);
   const GemmPlan plan = plan_gemm(rt, k, m, ws_bytes);
-  unsigned char* ws_split = static_cast<unsigned char*>(workspace) + x16_bytes(m, k);
-  cudaError_t e;
-  if (act_q8) {
-    e = launch_act_q8_f16(x, m, k, x16, status, stream);
-  } else {
-    const int64_t nvec = m * k / 8;
-    const int grid = static_cast<int>(std::min<int64_t>((nvec + 255) / 256,
-                                                        static_cast<int64_t>(device_sm_count()) * 8));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(std::max(grid, 1)), 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, bf16_to_f16_kernel, x, x16, nvec);
+  float* part = nullptr;
+  int* cnt = nullptr;
+  int ncnt = 0;
+  if (plan.nsplit > 1) {
+    unsigned char* p = static_cast<unsigned char*>(workspace) + x16_bytes(m, k);
+    part = reinterpret_cast<float*>(p);
+    cnt = reinterpret_cast<int*>(p + round256(static_cast<size_t>(plan.nsplit) * m * rt * kBM * 4));
+    ncnt = static_cast<int>(rt * ((m + plan.bn - 1) / plan.bn));
   }
+  cudaError_t e;
+  if (q == 4)
+    e = act_q8 ? run_x16<8, true>(x, x16, m, k, cnt, ncnt, status, stream)
+               : run_x16<8, false>(x, x16, m, k, cnt, ncnt, status, stream);
+  else
+    e = act_q8 ? run_x16<16, true>(x, x16, m, k, cnt, ncnt, status, stream)
+               : run_x16<16, false>(x, x16, m, k, cnt, ncnt, status, stream);
   if (e != cudaSuccess) return e;
-  const GemmCall c{ts, ys, count, x16, m, status, stream, plan, ws_split};
-  switch (ts[0]->q) {
+  const GemmCall c{ts, ys, count, x16, m, status, stream, plan, part, cnt};
+  switch (q) {
     case 2: return gemm_grid<2>(c);
     case 3: return gemm_grid<3>(c);
     case 4: return gemm_grid<4>(c);

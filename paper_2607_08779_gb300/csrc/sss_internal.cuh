@@ -57,8 +57,6 @@ cudaError_t launch_gemm_multi(const sss_qtensor_t* const* ts, float* const* ys, 
 
 cudaError_t launch_act_q8(const uint16_t* x, int64_t rows, int64_t k, int8_t* q, uint16_t* d,
                           uint32_t* status, cudaStream_t stream);
-cudaError_t launch_act_q8_f16(const uint16_t* x, int64_t rows, int64_t k, __half* out,
-                              uint32_t* status, cudaStream_t stream);
 
 cudaError_t launch_hadamard(const float* w, float* out, int64_t n, int64_t k, int b, int side,
                             cudaStream_t stream);
