@@ -85,6 +85,20 @@ __device__ __forceinline__ bool q_wait(uint32_t bar, uint32_t parity, volatile i
   }
 }
 
+// one bulk copy of `bytes` from global memory into shared memory, announced
+// on the mbarrier bar
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
+                                          uint64_t* bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(q_su32(bar)),
+               "r"(bytes)
+               : "memory");
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+      "[%3];" ::"r"(q_su32(dst)),
+      "l"(src), "r"(bytes), "r"(q_su32(bar))
+      : "memory");
+}
+
 // rotate the 64-bit value (hi:lo) left by n bits (0 <= n < 64)
 __device__ __forceinline__ void rotl64(uint32_t& lo, uint32_t& hi, int n) {
   uint32_t a = lo, b = hi;
@@ -336,15 +350,7 @@ __global__ void __launch_bounds__(kQThreads, 1)
         const int64_t w0 = (blockIdx.x + i * gridDim.x) * static_cast<int64_t>(kQChunk);
         const uint32_t bytes =
             static_cast<uint32_t>((nweights - w0 < kQChunk ? nweights - w0 : kQChunk) * 4);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
-                         q_su32(&full[s])),
-                     "r"(bytes)
-                     : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
-            "[%3];" ::"r"(q_su32(smem + s * kQChunk * 4)),
-            "l"(w + w0), "r"(bytes), "r"(q_su32(&full[s]))
-            : "memory");
+        bulk_load(smem + s * kQChunk * 4, w + w0, bytes, &full[s]);
         issued = i + 1;
       }
       if (*abort) {  // copies still in flight must land before the CTA exits
@@ -435,31 +441,6 @@ __device__ __forceinline__ void fwht_chunk(float* s, int b, int col) {
   }
 }
 
-// input side: out[r][c0 .. c0+b) = H_b w[r][c0 .. c0+b) / sqrt(b)
-__global__ void __launch_bounds__(kRotThreads)
-    hadamard_rows_kernel(const float* __restrict__ w, float* __restrict__ out, int64_t nweights,
-                         int b, float norm) {
-  __shared__ __align__(16) float s[kRotChunk];
-  const int64_t nchunks = (nweights + kRotChunk - 1) / kRotChunk;
-  for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const int64_t w0 = c * kRotChunk;
-    const int nv = static_cast<int>(nweights - w0 < kRotChunk ? nweights - w0 : kRotChunk);
-    for (int i = threadIdx.x; i < kRotChunk / 4; i += kRotThreads)
-      reinterpret_cast<float4*>(s)[i] =
-          4 * i < nv ? __ldcs(reinterpret_cast<const float4*>(w + w0) + i)
-                     : make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    fwht_chunk(s, b, 1);
-    for (int i = threadIdx.x; i < nv / 4; i += kRotThreads) {
-      float4 v = reinterpret_cast<float4*>(s)[i];
-      v.x = __fmul_rn(v.x, norm); v.y = __fmul_rn(v.y, norm);
-      v.z = __fmul_rn(v.z, norm); v.w = __fmul_rn(v.w, norm);
-      reinterpret_cast<float4*>(out + w0)[i] = v;
-    }
-    __syncthreads();
-  }
-}
-
 // output side: for every column, out[r0 .. r0+b)[c] = H_b w[r0 .. r0+b)[c] / sqrt(b);
 // a tile is b rows x C = 8192/b columns (16-byte accesses when C >= 4)
 __global__ void __launch_bounds__(kRotThreads)
@@ -497,46 +478,296 @@ __global__ void __launch_bounds__(kRotThreads)
   }
 }
 
-// The input-side rotation fused into the quantizer: each 8192-value chunk
-// is rotated in shared memory and quantized from there (the rotated fp32
-// weights never reach HBM).  Thread t owns run t of the chunk and reads it
-// in the rotated chunk order of the ring quantizer.
+// ---------------------------------------------------------------------------
+// Input side: out[r][c0 .. c0+b) = H_b w[r][c0 .. c0+b) / sqrt(b), written as
+// fp32 (sss_hadamard) or quantized from shared memory (sss_quantize_rotated:
+// the rotated fp32 weights never reach HBM).
+//
+// Persistent CTAs with the quantizer's ring: a producer thread streams chunks
+// of 8192 values into six 32 KB stages; three groups of four warps transform
+// them in place.  A thread holds 64 values at a time, as 32 packed pairs for
+// the two-wide fp32 instructions (each half rounds as the scalar one), and
+// runs six butterfly stages on them in registers: the strides 1 .. 32 on 64
+// consecutive values, then 64 .. 2048 on values 64 apart; stride 4096 (blocks
+// of 8192) is a pass of its own.  So the chunk crosses shared memory five
+// times for any block up to 4096, where a butterfly at a time crossed it
+// twelve times with an integer division each (4096: 418 us for 14336 x 4096
+// q = 3, 623 GB/s).
+// The pass over consecutive values reads the 16-byte pieces c of its 256 bytes
+// in the order c ^ (t & 7), which keeps a quarter-warp's banks distinct; a
+// butterfly between pieces then finds its lower element in either of two
+// slots, and a multiplier of +-1 in an FMA (exact product, one rounding) gives
+// the sum and the difference their sides without a select.
+// Bound by instruction issue and shared memory (about equal), then HBM.
+// ---------------------------------------------------------------------------
+
+constexpr int kRGroups = 3;   // divides the stages: each group has its own (see q_wait's parity)
+constexpr int kRThreads = 32 + 128 * kRGroups;
+static_assert(kQStages % kRGroups == 0, "a group waits for every phase of its stages");
+
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// the butterflies between pairs p and p + D (a multiple of pairs apart)
+template <int D>
+__device__ __forceinline__ void stage2(uint64_t (&v)[32], uint64_t neg1) {
+#pragma unroll
+  for (int p = 0; p < 32; ++p)
+    if ((p & D) == 0) {
+      const uint64_t a = v[p], c = v[p + D];
+      v[p] = add2(a, c);
+      v[p + D] = fma2(neg1, c, a);
+    }
+}
+// the same where pair p holds the upper element when s = (-1, -1); n = -s
+template <int D>
+__device__ __forceinline__ void stage2_signed(uint64_t (&v)[32], uint64_t s, uint64_t n) {
+#pragma unroll
+  for (int p = 0; p < 32; ++p)
+    if ((p & D) == 0) {
+      const uint64_t a = v[p], c = v[p + D];
+      v[p] = fma2(s, a, c);
+      v[p + D] = fma2(n, c, a);
+    }
+}
+// the butterflies inside every pair
+__device__ __forceinline__ void stage1(uint64_t (&v)[32]) {
+#pragma unroll
+  for (int p = 0; p < 32; ++p) {
+    float a, c;
+    unpack2(v[p], a, c);
+    v[p] = pack2(__fadd_rn(a, c), __fsub_rn(a, c));
+  }
+}
+
+__device__ __forceinline__ void group_sync(int g) {
+  asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
+}
+
+// The first lb stages of the transform of the chunk at shared address `base`,
+// by the 128 threads t of group g; ends with a barrier of the group.
+__device__ __forceinline__ void fwht_regs(uint32_t base, int lb, int t, int g) {
+  const uint64_t neg1 = pack2(-1.f, -1.f), pos1 = pack2(1.f, 1.f);
+  uint64_t v[32];
+  {
+    const uint32_t r = static_cast<uint32_t>(t) & 7u;
+    const uint32_t mine = base + 256u * static_cast<uint32_t>(t);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const uint32_t c = (j & 8) | ((j ^ r) & 7u);
+      asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
+                   : "=l"(v[2 * j]), "=l"(v[2 * j + 1])
+                   : "r"(mine + 16u * c));
+    }
+    if (lb > 0) stage1(v);
+    if (lb > 1) stage2<1>(v, neg1);
+    if (lb > 2) stage2_signed<2>(v, (r & 1u) ? neg1 : pos1, (r & 1u) ? pos1 : neg1);
+    if (lb > 3) stage2_signed<4>(v, (r & 2u) ? neg1 : pos1, (r & 2u) ? pos1 : neg1);
+    if (lb > 4) stage2_signed<8>(v, (r & 4u) ? neg1 : pos1, (r & 4u) ? pos1 : neg1);
+    if (lb > 5) stage2<16>(v, neg1);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const uint32_t c = (j & 8) | ((j ^ r) & 7u);
+      asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(mine + 16u * c), "l"(v[2 * j]),
+                   "l"(v[2 * j + 1])
+                   : "memory");
+    }
+  }
+  group_sync(g);
+  if (lb <= 6) return;
+  {
+    // values 64 apart: element i of the thread is 64 i + (t & 63) of its half
+    const uint32_t mine = base + 4u * static_cast<uint32_t>(t & 63) + 16384u * (t >> 6);
+#pragma unroll
+    for (int p = 0; p < 32; ++p) {
+      float a, c;
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(mine + 512u * p));
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(c) : "r"(mine + 512u * p + 256u));
+      v[p] = pack2(a, c);
+    }
+    stage1(v);
+    if (lb > 7) stage2<1>(v, neg1);
+    if (lb > 8) stage2<2>(v, neg1);
+    if (lb > 9) stage2<4>(v, neg1);
+    if (lb > 10) stage2<8>(v, neg1);
+    if (lb > 11) stage2<16>(v, neg1);
+#pragma unroll
+    for (int p = 0; p < 32; ++p) {
+      float a, c;
+      unpack2(v[p], a, c);
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(mine + 512u * p), "f"(a) : "memory");
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(mine + 512u * p + 256u), "f"(c) : "memory");
+    }
+  }
+  group_sync(g);
+  if (lb <= 12) return;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const uint32_t lo = base + 16u * static_cast<uint32_t>(t + 128 * j);
+    uint64_t a0, a1, c0, c1;
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a0), "=l"(a1) : "r"(lo));
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(c0), "=l"(c1) : "r"(lo + 16384u));
+    asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(lo), "l"(add2(a0, c0)),
+                 "l"(add2(a1, c1))
+                 : "memory");
+    asm volatile("st.shared.v2.b64 [%0], {%1, %2};" ::"r"(lo + 16384u), "l"(fma2(neg1, c0, a0)),
+                 "l"(fma2(neg1, c1, a1))
+                 : "memory");
+  }
+  group_sync(g);
+}
+
+// The ring around fwht_regs: final(base, nv, w0, t) takes each transformed
+// chunk of nv values from shared memory, w0 its first value.
+template <class Final>
+__device__ __forceinline__ void rotate_rows_ring(const float* __restrict__ w, int64_t nweights,
+                                                 int lb, uint32_t* __restrict__ status,
+                                                 Final final) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kQStages * kQChunk * 4);
+  uint64_t* empty = full + kQStages;
+  volatile int* abort = reinterpret_cast<volatile int*>(empty + kQStages);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t nchunks = (nweights + kQChunk - 1) / kQChunk;
+  // this CTA's chunks: blockIdx.x + i * gridDim.x, i = 0 .. my - 1
+  const int64_t my =
+      blockIdx.x < nchunks ? (nchunks - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kQStages; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(q_su32(&full[s])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;" ::"r"(q_su32(&empty[s])) : "memory");
+    }
+    *abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // a programmatic dependent launch, as quantize_kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) {
+    if (lane == 0) {
+      int64_t issued = 0;
+      for (int64_t i = 0; i < my; ++i) {
+        const int s = static_cast<int>(i % kQStages);
+        if (!q_wait(q_su32(&empty[s]), (static_cast<uint32_t>(i / kQStages) & 1u) ^ 1u, abort))
+          break;
+        const int64_t w0 = (blockIdx.x + i * gridDim.x) * static_cast<int64_t>(kQChunk);
+        bulk_load(smem + s * kQChunk * 4, w + w0,
+                  static_cast<uint32_t>((nweights - w0 < kQChunk ? nweights - w0 : kQChunk) * 4),
+                  &full[s]);
+        issued = i + 1;
+      }
+      if (*abort) {  // copies still in flight must land before the CTA exits
+        int drain = 0;
+        for (int64_t i = issued > kQStages ? issued - kQStages : 0; i < issued; ++i)
+          (void)q_wait(q_su32(&full[i % kQStages]), static_cast<uint32_t>(i / kQStages) & 1u,
+                       &drain);
+      }
+    }
+  } else {
+    const int g = (warp - 1) >> 2;
+    const int t = static_cast<int>(threadIdx.x) - 32 - 128 * g;
+    for (int64_t i = g; i < my; i += kRGroups) {
+      const int s = static_cast<int>(i % kQStages);
+      // one verdict for the group: its barriers need all four warps
+      const bool got = q_wait(q_su32(&full[s]), static_cast<uint32_t>(i / kQStages) & 1u, abort);
+      uint32_t bad;
+      asm volatile(
+          "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred p, %2, 128, q;\n"
+          " selp.u32 %0, 1, 0, p;\n}\n"
+          : "=r"(bad)
+          : "r"(got ? 0u : 1u), "r"(1 + g)
+          : "memory");
+      if (bad) break;
+      const int64_t w0 = (blockIdx.x + i * gridDim.x) * static_cast<int64_t>(kQChunk);
+      const int nv = static_cast<int>(nweights - w0 < kQChunk ? nweights - w0 : kQChunk);
+      const uint32_t base = q_su32(smem + s * kQChunk * 4);
+      // (values past nv are leftovers; no butterfly crosses into the nv)
+      fwht_regs(base, lb, t, g);
+      final(base, nv, w0, t);
+      // the stage goes back to the copies: this thread's accesses first
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(q_su32(&empty[s]))
+                     : "memory");
+    }
+  }
+  __syncthreads();
+  if (*abort && threadIdx.x == 0 && status != nullptr) atomicOr(status, SSS_FLAG_TIMEOUT);
+}
+
+__global__ void __launch_bounds__(kRThreads, 1)
+    hadamard_rows_kernel(const float* __restrict__ w, float* __restrict__ out, int64_t nweights,
+                         int lb, float norm) {
+  rotate_rows_ring(w, nweights, lb, nullptr, [&](uint32_t base, int nv, int64_t w0, int t) {
+    for (int i = t; i < nv / 4; i += 128) {
+      float4 v;
+      asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+                   : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                   : "r"(base + 16u * static_cast<uint32_t>(i)));
+      v.x = __fmul_rn(v.x, norm); v.y = __fmul_rn(v.y, norm);
+      v.z = __fmul_rn(v.z, norm); v.w = __fmul_rn(v.w, norm);
+      reinterpret_cast<float4*>(out + w0)[i] = v;
+    }
+  });
+}
+
+// Threads t of a group own runs t and t + 128 of the chunk, read in the
+// rotated order of the quantizer.
 template <int Q, int GRID, int G, bool STATS>
-__global__ void __launch_bounds__(kRotThreads)
-    rotate_quantize_kernel(const float* __restrict__ w, int64_t nweights, int b, float norm,
+__global__ void __launch_bounds__(kRThreads, 1)
+    rotate_quantize_kernel(const float* __restrict__ w, int64_t nweights, int lb, float norm,
                            uint8_t* __restrict__ codes, uint16_t* __restrict__ scales,
                            uint16_t* __restrict__ mins, uint8_t* __restrict__ clip,
                            uint32_t* __restrict__ status) {
-  __shared__ __align__(16) float s[kRotChunk];
-  const int64_t nchunks = (nweights + kRotChunk - 1) / kRotChunk;
-  const int sl = threadIdx.x, r = sl & 7;
-  for (int64_t c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const int64_t w0 = c * kRotChunk;
-    const int nv = static_cast<int>(nweights - w0 < kRotChunk ? nweights - w0 : kRotChunk);
-    for (int i = threadIdx.x; i < kRotChunk / 4; i += kRotThreads)
-      reinterpret_cast<float4*>(s)[i] =
-          4 * i < nv ? __ldcs(reinterpret_cast<const float4*>(w + w0) + i)
-                     : make_float4(0.f, 0.f, 0.f, 0.f);
-    __syncthreads();
-    fwht_chunk(s, b, 1);
-    const bool valid = 32 * sl < nv;
-    float x[32];
-    const float4* run = reinterpret_cast<const float4*>(s + 32 * sl);
+  rotate_rows_ring(w, nweights, lb, status, [&](uint32_t base, int nv, int64_t w0, int t) {
+    const int r = t & 7;
+#pragma unroll 1
+    for (int sl = t; sl < kQChunk / 32; sl += 128) {
+      const bool valid = 32 * sl < nv;
+      const uint32_t run_a = base + 128u * static_cast<uint32_t>(sl);
+      float x[32];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float4 v = run[(j + r) & 7];
-      x[4 * j] = __fmul_rn(v.x, norm); x[4 * j + 1] = __fmul_rn(v.y, norm);
-      x[4 * j + 2] = __fmul_rn(v.z, norm); x[4 * j + 3] = __fmul_rn(v.w, norm);
+      for (int j = 0; j < 8; ++j) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (valid)
+          asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+                       : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                       : "r"(run_a + 16u * static_cast<uint32_t>((j + r) & 7)));
+        x[4 * j] = __fmul_rn(v.x, norm); x[4 * j + 1] = __fmul_rn(v.y, norm);
+        x[4 * j + 2] = __fmul_rn(v.z, norm); x[4 * j + 3] = __fmul_rn(v.w, norm);
+      }
+      quantize_run<Q, GRID, G, STATS>(
+          x,
+          [&](int e) {
+            float v = 0.f;
+            if (valid)
+              asm volatile("ld.shared.f32 %0, [%1];"
+                           : "=f"(v)
+                           : "r"(run_a + 16u * static_cast<uint32_t>(((e >> 2) + r) & 7) +
+                                 4u * static_cast<uint32_t>(e & 3)));
+            return __fmul_rn(v, norm);
+          },
+          r, valid, w0 / 32 + sl, codes, scales, mins, clip, status);
     }
-    quantize_run<Q, GRID, G, STATS>(
-        x,
-        [&](int e) {
-          return __fmul_rn(reinterpret_cast<const float*>(run)[4 * (((e >> 2) + r) & 7) + (e & 3)],
-                           norm);
-        },
-        r, valid, w0 / 32 + sl, codes, scales, mins, clip, status);
-    __syncthreads();  // the chunk is read: the next one may overwrite it
-  }
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -706,19 +937,41 @@ cudaError_t dequant_dispatch_grid(const sss_qtensor_t& t, void* out, int dtype,
   return dequant_dispatch_out<Q, SSS_GRID_SIGNED_SYM>(t, out, dtype, stream);
 }
 
+// a kernel around rotate_rows_ring: one CTA per SM, a programmatic dependent
+// launch
+template <class K, class... A>
+cudaError_t launch_ring(K kern, int threads, int64_t nweights, cudaStream_t stream, A... args) {
+  cudaError_t e = ensure_smem(kern, kQSmem);
+  if (e != cudaSuccess) return e;
+  const int64_t nchunks = (nweights + kQChunk - 1) / kQChunk;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(std::min<int64_t>(device_sm_count(), nchunks)), 1, 1);
+  cfg.blockDim = dim3(static_cast<unsigned>(threads), 1, 1);
+  cfg.dynamicSmemBytes = kQSmem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+int log2_of(int b) {
+  int lb = 0;
+  while ((1 << lb) < b) ++lb;
+  return lb;
+}
+
 template <int Q, int GRID, int G>
 cudaError_t rotq_dispatch(const float* w, int b, float norm, const sss_qtensor_t& t,
                           uint8_t* clip, uint32_t* status, cudaStream_t stream) {
   const int64_t nweights = t.n * t.k;
-  const int64_t nchunks = (nweights + kRotChunk - 1) / kRotChunk;
-  const int grid = static_cast<int>(std::min<int64_t>(device_sm_count() * 8, nchunks));
   if (clip != nullptr)
-    rotate_quantize_kernel<Q, GRID, G, true><<<grid, kRotThreads, 0, stream>>>(
-        w, nweights, b, norm, t.codes, t.scales, t.mins, clip, status);
-  else
-    rotate_quantize_kernel<Q, GRID, G, false><<<grid, kRotThreads, 0, stream>>>(
-        w, nweights, b, norm, t.codes, t.scales, t.mins, clip, status);
-  return cudaGetLastError();
+    return launch_ring(rotate_quantize_kernel<Q, GRID, G, true>, kRThreads, nweights, stream, w,
+                       nweights, log2_of(b), norm, t.codes, t.scales, t.mins, clip, status);
+  return launch_ring(rotate_quantize_kernel<Q, GRID, G, false>, kRThreads, nweights, stream, w,
+                     nweights, log2_of(b), norm, t.codes, t.scales, t.mins, clip, status);
 }
 
 template <int Q, int GRID>
@@ -755,9 +1008,8 @@ cudaError_t launch_hadamard(const float* w, float* out, int64_t n, int64_t k, in
                             cudaStream_t stream) {
   const int sms = device_sm_count();
   if (side == 0) {
-    const int64_t nchunks = (n * k + kRotChunk - 1) / kRotChunk;
-    const int grid = static_cast<int>(std::min<int64_t>(sms * 8, nchunks));
-    hadamard_rows_kernel<<<grid, kRotThreads, 0, stream>>>(w, out, n * k, b, hadamard_norm(b));
+    return launch_ring(hadamard_rows_kernel, kRThreads, n * k, stream, w, out, n * k, log2_of(b),
+                       hadamard_norm(b));
   } else {
     const int64_t tiles = (n / b) * (k / (kRotChunk / b));
     const int grid = static_cast<int>(std::min<int64_t>(sms * 8, tiles));
