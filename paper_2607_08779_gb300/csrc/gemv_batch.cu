@@ -1,5 +1,7 @@
 // gemv_batch.cu -- decode GEMV for batches of 2..16 activation vectors over
-// packed q-bit codes (sm_103a), the batched path of sss_gemv.
+// packed q-bit codes (sm_103a), the batched path of sss_gemv for q = 3 (whose
+// two bit planes per group do not fall into the words that gemv_cluster.cu
+// hands its quads) and for a k whose staged x fits no cluster.
 //
 // y[b][r] = sum_k w^[r][k] x[b][k] with w^ the dequantised weight of
 // eq:quantizer (Appendix B.3 product).  Unlike the batch-1 kernels, the

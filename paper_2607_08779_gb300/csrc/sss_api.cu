@@ -197,14 +197,21 @@ sss_status_t sss_gemv(const sss_qtensor_t* qt, const uint16_t* x_bf16, int32_t b
                   cudaMemsetAsync(y, 0, sizeof(float) * static_cast<size_t>(batch) * qt->n,
                                   static_cast<cudaStream_t>(stream)));
   }
-  // batch 1: the streaming kernel; batch 2..16: the batched kernel (fp16
-  // weight operand); shapes neither takes (k not a multiple of 256,
+  // batch 1: the streaming kernel; batch 2..16: the cluster kernel for q = 2
+  // and 4 (a Llama3-8B layer's seven matrices, q = 4 at batch 4: 54 us against
+  // 70 us), the batched kernel (fp16 weight operand) for q = 3 and a k whose
+  // staged x fits no cluster; shapes none takes (k not a multiple of 256,
   // unaligned buffers): the general kernel
   if (batch == 1 && gemv_stream_eligible(*qt, x_bf16)) {
     const sss_qtensor_t* one[1] = {qt};
     float* yy[1] = {y};
     return finish("sss_gemv", launch_gemv_stream(one, yy, 1, x_bf16, 0u, dev_status,
                                                  static_cast<cudaStream_t>(stream)));
+  }
+  if (batch >= 2 && gemv_cluster_eligible(*qt, x_bf16, batch, y)) {
+    const cudaError_t e = launch_gemv_cluster(*qt, x_bf16, batch, y, dev_status,
+                                              static_cast<cudaStream_t>(stream));
+    if (e != cudaErrorNotSupported) return finish("sss_gemv", e);
   }
   if (batch >= 2 && gemv_batch_eligible(*qt, x_bf16, batch, y)) {
     return finish("sss_gemv", launch_gemv_batch(*qt, x_bf16, batch, y, dev_status,

@@ -43,6 +43,10 @@ bool gemv_batch_eligible(const sss_qtensor_t& t, const uint16_t* x, int batch, c
 cudaError_t launch_gemv_batch(const sss_qtensor_t& t, const uint16_t* x, int batch, float* y,
                               uint32_t* status, cudaStream_t stream);
 
+bool gemv_cluster_eligible(const sss_qtensor_t& t, const uint16_t* x, int batch, const float* y);
+cudaError_t launch_gemv_cluster(const sss_qtensor_t& t, const uint16_t* x, int batch, float* y,
+                                uint32_t* status, cudaStream_t stream);
+
 // matrices of one sss_gemm_multi call (sharing X)
 constexpr int kMaxGemmJobs = 4;
 size_t gemm_workspace_bytes(const sss_qtensor_t& t, int64_t m);
