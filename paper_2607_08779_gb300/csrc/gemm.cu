@@ -622,11 +622,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // Launched as a programmatic dependent launch: the set-up above (barriers,
-  // tensor memory) overlaps the preceding kernel's drain; nothing in global
-  // memory is read or written before that kernel has completed.
+  // Launched as a programmatic dependent launch of x16_kernel, which releases
+  // it only once everything before that kernel has completed.  So the packed
+  // weights and scales may be read at once; what x16_kernel writes (X, the
+  // split counters), and every write of this kernel, waits for it: the
+  // producer before its first activation tile, the other warps before their
+  // first epilogue.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
 
   if (warp == 0) {
     // ---------------- TMA producer: activation and code tiles ----------------
@@ -660,6 +662,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // code tiles run one ahead of the activations: their codes have the
       // dequantisation before them
       ok = nw == 0 || put_w(0);
+      if (xn == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
       for (int p = 0; p < w.nsteps && ok; ++p) {
         if (p % 2 == 0 && p / 2 + 1 < nw && !put_w(p / 2 + 1)) {
           ok = false;
@@ -846,18 +849,24 @@ __global__ void __launch_bounds__(kThreads, 1)
             return;
           }
           load_tile_codes<Q>(smem_u32(smem) + S::W_OFF + ws * S::W_BYTES, row_i, p & 1, wv);
-          // the codes are in registers before the TMA may overwrite the tile
-          // (without the fence the loads can still be in flight at the arrive)
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&empty_w[ws]);
         } else {
 #pragma unroll
           for (int i = 0; i < 4 * Q; ++i) wv[i] = wn[i];
         }
         order_codes<Q>(wv, a.G, codes);
       }
-      if (p >= w.nsteps) return;
+      // hands the code tile back: after the codes have been used, since an
+      // arrive right behind the loads lets the TMA overwrite rows whose loads
+      // are still in flight
+      auto release_w = [&]() {
+        if constexpr (CT) {
+          if (lane == 0) mbar_arrive(&empty_w[((P + p) >> 1) % WS]);
+        }
+      };
+      if (p >= w.nsteps) {  // (no codes were used: nothing to overwrite)
+        release_w();
+        return;
+      }
       fetch(p + 4);
       if constexpr (!ASYM)
         smax = __hmax2(smax, __hmax2(__habs2(*reinterpret_cast<const __half2*>(&sv.x)),
@@ -896,6 +905,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // (sss_test_set_stall: warp 2 leaves the first stage one arrive short,
       // so the MMA issuer's wait for it runs out)
       if (lane == 0 && !(a.stall && first && p == 0 && warp == 2)) mbar_arrive(&full_a[slot]);
+      release_w();
     };
 
     int n = 0;
@@ -916,6 +926,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // ---- epilogue of item e = it: a warp may read tensor-memory lanes
       // 32*(warp % 4) .. +31; the four groups take alternate sets of 32 columns
+      if (n == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
       const int buf = n % NB;
       const bool fin = ok && mbar_wait(&done[buf], static_cast<uint32_t>(n / NB) & 1u, abort);
       ok = __all_sync(0xffffffffu, fin);  // warp-uniform: tcgen05.ld is .sync.aligned
@@ -963,6 +974,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (__any_sync(0xffffffffu, big) && lane == 0 && a.status != nullptr)
       atomicOr(a.status, SSS_FLAG_RANGE);
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // (a CTA whose wait ran out, too)
 
   tc_fence_before();
   __syncthreads();
@@ -986,9 +998,10 @@ __global__ void __launch_bounds__(256)
     x16_kernel(const uint16_t* __restrict__ x, __half* __restrict__ y, int64_t nvec,
                int* __restrict__ cnt, int ncnt, uint32_t* __restrict__ status) {
   // programmatic dependent launch: start once the preceding kernel (which
-  // may still read the fp16 buffer) has completed
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // may still read the fp16 buffer) has completed, and only then let the GEMM
+  // start, which reads the weights before this kernel has ended
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   for (int64_t i = t0; i < ncnt; i += stride) cnt[i] = 0;
