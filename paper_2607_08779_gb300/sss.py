@@ -81,6 +81,8 @@ def library_path() -> str:
 def load(build_if_needed: bool = True):
     """Load libsss.so (building it with nvcc first if it is missing/stale)."""
     global _lib
+    if _lib is not None:  # set once, complete
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -138,14 +140,15 @@ def load(build_if_needed: bool = True):
 
 
 def _ptr(t) -> int:
-    return 0 if t is None else int(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def _stream(stream) -> int:
     import torch
 
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the raw handle of the current stream, without building a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(stream.cuda_stream)
 
 
@@ -176,6 +179,39 @@ def _on_device(fn: str, **tensors):
     for name, t in tensors.items():
         if t is not None and not getattr(t, "is_cuda", False):
             raise SssError(fn, 1, f"{name} must be a CUDA tensor")
+
+
+def _plain(t, dtype, numel) -> bool:
+    """Whether t passes _need and _on_device, as one expression: a call that is
+    in order is checked here, and only another one goes through them, check by
+    check, for the error it raises."""
+    return (t is not None and t.dtype is dtype and t.is_cuda and t.is_contiguous()
+            and t.numel() == numel)
+
+
+def _plain_qtensor(qt: "QTensor") -> bool:
+    import torch
+
+    if qt.group <= 0:
+        return False
+    ng = qt.n * (qt.k // qt.group)
+    return (_plain(qt.codes, torch.uint8, qt.n * qt.k * qt.q // 8)
+            and _plain(qt.scales, torch.int16, ng)
+            and (qt.mins is None and qt.grid != GRID_ASYM or _plain(qt.mins, torch.int16, ng)))
+
+
+def _plain_status(dev_status) -> bool:
+    import torch
+
+    return dev_status is None or (dev_status.dtype is torch.int32 and dev_status.is_cuda
+                                  and dev_status.is_contiguous() and dev_status.numel() >= 1)
+
+
+def _plain_workspace(workspace) -> bool:
+    import torch
+
+    return workspace is None or (workspace.dtype is torch.uint8 and workspace.is_cuda
+                                 and workspace.is_contiguous())
 
 
 def _need_qtensor(fn: str, qt: "QTensor"):
@@ -257,12 +293,14 @@ def sss_quantize(w, q: int, group: int, grid: int, out: Optional[QTensor] = None
         out = empty_qtensor(n, k, q, group, grid, device=w.device)
     if (out.n, out.k, out.q, out.group, out.grid) != (n, k, q, group, grid):
         raise SssError("sss_quantize", 1, "out does not match w's shape, q, group and grid")
-    _need_qtensor("sss_quantize", out)
-    if clip_counts is not None and group > 0:
-        _need("sss_quantize", "clip_counts", clip_counts, torch.uint8, n * (k // group) * 2)
-    _need_status("sss_quantize", dev_status)
-    _on_device("sss_quantize", w=w, codes=out.codes, scales=out.scales, mins=out.mins,
-               clip_counts=clip_counts, dev_status=dev_status)
+    if not (clip_counts is None and w.is_cuda and _plain_qtensor(out)
+            and _plain_status(dev_status)):
+        _need_qtensor("sss_quantize", out)
+        if clip_counts is not None and group > 0:
+            _need("sss_quantize", "clip_counts", clip_counts, torch.uint8, n * (k // group) * 2)
+        _need_status("sss_quantize", dev_status)
+        _on_device("sss_quantize", w=w, codes=out.codes, scales=out.scales, mins=out.mins,
+                   clip_counts=clip_counts, dev_status=dev_status)
     d = out.desc()
     st = load().sss_quantize(_ptr(w), ctypes.byref(d), _ptr(clip_counts), _ptr(dev_status),
                              _stream(stream))
@@ -292,15 +330,17 @@ def sss_gemv(qt: QTensor, x, y=None, workspace=None, dev_status=None, stream=Non
     import torch
 
     batch = x.shape[0] if x.dim() == 2 else 1
-    _need("sss_gemv", "x", x, torch.bfloat16, batch * qt.k)
-    if y is None:
-        y = torch.empty((batch, qt.n), dtype=torch.float32, device=x.device)
-    _need("sss_gemv", "y", y, torch.float32, batch * qt.n)
-    _need_qtensor("sss_gemv", qt)
-    _need("sss_gemv", "workspace", workspace, torch.uint8, optional=True)
-    _need_status("sss_gemv", dev_status)
-    _on_device("sss_gemv", x=x, y=y, codes=qt.codes, scales=qt.scales, mins=qt.mins,
-               workspace=workspace, dev_status=dev_status)
+    if not (_plain(x, torch.bfloat16, batch * qt.k) and _plain(y, torch.float32, batch * qt.n)
+            and _plain_qtensor(qt) and _plain_workspace(workspace) and _plain_status(dev_status)):
+        _need("sss_gemv", "x", x, torch.bfloat16, batch * qt.k)
+        if y is None:
+            y = torch.empty((batch, qt.n), dtype=torch.float32, device=x.device)
+        _need("sss_gemv", "y", y, torch.float32, batch * qt.n)
+        _need_qtensor("sss_gemv", qt)
+        _need("sss_gemv", "workspace", workspace, torch.uint8, optional=True)
+        _need_status("sss_gemv", dev_status)
+        _on_device("sss_gemv", x=x, y=y, codes=qt.codes, scales=qt.scales, mins=qt.mins,
+                   workspace=workspace, dev_status=dev_status)
     d = qt.desc()
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     st = load().sss_gemv(ctypes.byref(d), _ptr(x), batch, _ptr(y), _ptr(workspace), ws_bytes,
@@ -338,15 +378,17 @@ def _gemm(fn: str, qt: QTensor, x, y, workspace, dev_status, stream):
     import torch
 
     m = x.shape[0]
-    _need(fn, "x", x, torch.bfloat16, m * qt.k)
-    if y is None:
-        y = torch.empty((m, qt.n), dtype=torch.float32, device=x.device)
-    _need(fn, "y", y, torch.float32, m * qt.n)
-    _need_qtensor(fn, qt)
-    _need(fn, "workspace", workspace, torch.uint8, optional=True)
-    _need_status(fn, dev_status)
-    _on_device(fn, x=x, y=y, codes=qt.codes, scales=qt.scales, mins=qt.mins,
-               workspace=workspace, dev_status=dev_status)
+    if not (_plain(x, torch.bfloat16, m * qt.k) and _plain(y, torch.float32, m * qt.n)
+            and _plain_qtensor(qt) and _plain_workspace(workspace) and _plain_status(dev_status)):
+        _need(fn, "x", x, torch.bfloat16, m * qt.k)
+        if y is None:
+            y = torch.empty((m, qt.n), dtype=torch.float32, device=x.device)
+        _need(fn, "y", y, torch.float32, m * qt.n)
+        _need_qtensor(fn, qt)
+        _need(fn, "workspace", workspace, torch.uint8, optional=True)
+        _need_status(fn, dev_status)
+        _on_device(fn, x=x, y=y, codes=qt.codes, scales=qt.scales, mins=qt.mins,
+                   workspace=workspace, dev_status=dev_status)
     d = qt.desc()
     if workspace is None:
         need = int(load().sss_workspace_bytes(ctypes.byref(d), m, OP_GEMM))
