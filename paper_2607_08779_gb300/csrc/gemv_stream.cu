@@ -39,6 +39,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "act_q8.cuh"
 #include "gemv_common.cuh"
@@ -79,19 +80,18 @@ __device__ __forceinline__ void field_desc(int p, int& ea, int& eb, int& pos) {
   }
 }
 
-// the high-plane bits of elements 16w .. 16w+15 (w = word of the sub-chunk)
-// spread to every other bit: element 16w+e at bit 2e (e < 8) and element
-// 16w+8+e at bit 16+2e
-__device__ __forceinline__ uint32_t spread_high(uint32_t hi_plane, int w) {
-  uint32_t x = __byte_perm(hi_plane, 0u, w ? 0x4342u : 0x4140u);
-  x = (x | (x << 4)) & 0x0F0F0F0Fu;
-  x = (x | (x << 2)) & 0x33333333u;
-  x = (x | (x << 1)) & 0x55555555u;
-  return x;
+// Bits of the high plane (q=3) of elements 16w+e and 16w+8+e at bits e and 16+e
+// (w = word of the sub-chunk).
+__device__ __forceinline__ uint32_t high_halves(uint32_t hi_plane, int w) {
+  return __byte_perm(hi_plane, 0u, w ? 0x4342u : 0x4140u);
 }
 
 // Operand of pair p.  w[0..3] (q=4), w[0..1] (q=2) or w[0..1] + the high
-// plane w[2] (q=3) of one sub-chunk; hs[0..1] = spread_high of w[2] for q=3.
+// plane w[2] (q=3) of one sub-chunk; for q=3 hs[0..1] = high_halves of w[2] and
+// hs[2..3] the same shifted down by 3.  A field's high bit is one left shift
+// from its place at pos + 2 (the multiply-add pipe takes left shifts, and the
+// logic pipe is the one that bounds this kernel; spreading the plane to every
+// other bit first took three more logic instructions per word).
 template <int Q>
 __device__ __forceinline__ uint32_t field_pair(const uint32_t* w, const uint32_t* hs, int p) {
   if constexpr (Q == 4) {
@@ -105,8 +105,9 @@ __device__ __forceinline__ uint32_t field_pair(const uint32_t* w, const uint32_t
     if constexpr (Q == 2) {
       return lo;
     } else {
-      // high bit of element e at 2e in hs; wanted at pos + 2
-      const uint32_t h = e < 5 ? (hs[wi] << 2) : (hs[wi] >> 8);
+      // high bit of element e at bit e, wanted at pos + 2: up by e + 2, or from
+      // bit e - 3 up by e - 5
+      const uint32_t h = e < 5 ? (hs[wi] << (e + 2)) : (hs[2 + wi] << (e - 5));
       return lo | (h & (0x00040004u << pos));
     }
   }
@@ -119,9 +120,10 @@ __device__ __forceinline__ uint32_t field_pair(const uint32_t* w, const uint32_t
 // keeps every element exact in fp16 whatever the activations' magnitude.
 // sbf[i] = {b_i, f_i}: f_i = 2^(24 - E_i) undoes both scalings in the
 // epilogue, and b_i is the row-sum term of Appendix B.3 on the mma's scale:
-// sum(x) * 2^(E_i - 24), times -2^(q-1) for the symmetric grids.  Two
-// threads share a sub-chunk (16 elements each); threads tid = 0 ..
-// nthreads-1 (nthreads even) share the work; the caller synchronises.
+// sum(x) * 2^(E_i - 24), times -2^(q-1) for the symmetric grids.  Four
+// threads share a sub-chunk (8 elements each: at k = 4096 every thread of the
+// CTA has one part); threads tid = 0 .. nthreads-1 (whole warps) share the
+// work; the caller synchronises.
 //
 // With act_q8 the activations are first quantized to Q8_0 (act_q8.cuh; a
 // sub-chunk is one Q8_0 block): the staged operand is the int8 code q
@@ -228,7 +230,7 @@ struct StreamJob {
   const uint16_t* mins;
   float* y;
   int64_t n;
-  int64_t tile0;  // first global tile index of this job
+  int tile0;  // first global tile index of this job
 };
 
 struct StreamArgs {
@@ -236,7 +238,7 @@ struct StreamArgs {
   int njobs;
   const uint16_t* x;  // bf16 [k]
   int64_t k;
-  int64_t ntiles;
+  int ntiles;
   int lgkw;            // log2(warps per tile)
   int early_weights;   // prefetch weights before the grid-dependency wait
   int act_q8;          // quantize the activations to Q8_0 while staging them
@@ -251,8 +253,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
 
   const int nsc = static_cast<int>(a.k / 32);  // 32-code sub-chunks per row
   const int nunits = nsc / 8;                  // units of 256 codes
-  const int64_t nG = a.k / G;
-  const int64_t row_bytes = a.k * Q / 8;
+  // (32-bit, for 32 x 32 -> 64-bit multiplies: k < 2^31, and n is at most 2^31)
+  const int nG = static_cast<int>(a.k / G);
+  const int row_bytes = static_cast<int>(a.k * Q / 8);
   const int lgkw = a.lgkw;
   const int KW = 1 << lgkw;                    // warps per tile
   const int ngrp = kWarps >> lgkw;             // tiles in flight per CTA
@@ -281,16 +284,19 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
   // i = 0, 1, ... (consecutive tiles go to different SMs, so every SM gets
   // within one tile of the same work), and in each tile the units u = kw,
   // kw + KW, ... ----
-  const int64_t tstride = static_cast<int64_t>(gridDim.x) * ngrp;
-  const int64_t tfirst = static_cast<int64_t>(grp) * gridDim.x + blockIdx.x;
-  const int64_t my_tiles = tfirst < a.ntiles ? (a.ntiles - tfirst + tstride - 1) / tstride : 0;
+  // (32-bit: the host keeps the tile count to 2^30; of a group's a.rounds
+  // tiles only the last may be past the end)
+  const int grid = static_cast<int>(gridDim.x);
+  const int tstride = grid * ngrp;
+  const int tfirst = grp * grid + static_cast<int>(blockIdx.x);
+  const int my_tiles = a.rounds - (tfirst + (a.rounds - 1) * tstride >= a.ntiles ? 1 : 0);
   const bool has_units = kw < nunits;
 
   // This warp's flat unit stream: unit k is unit u = kw + (k % upw) * KW of
   // its i = k / upw-th tile, upw = units per tile for this warp (the host
   // keeps every count below 2^31).
   const int upw = has_units ? (nunits - kw + KW - 1) >> lgkw : 0;
-  const int total = static_cast<int>(my_tiles) * upw;
+  const int total = my_tiles * upw;
 
   constexpr int UB = 32 * Q;    // code bytes of one row in one unit
   constexpr int SPU = 256 / G;  // scales of one row in one unit
@@ -306,28 +312,29 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
 
   // the code/scale/min pointers of rows g and g+8 of this warp's i-th tile,
   // at its first unit
-  auto tile_ptrs = [&](int64_t i, const uint8_t** c, const uint16_t** sc, const uint16_t** mn) {
-    const int64_t t = tfirst + i * tstride;
+  auto tile_ptrs = [&](int i, const uint8_t** c, const uint16_t** sc, const uint16_t** mn) {
+    const int t = tfirst + i * tstride;
     int j = 0;
     while (j + 1 < a.njobs && t >= a.job[j + 1].tile0) ++j;
     const StreamJob& jb = a.job[j];
-    const int64_t row0 = (t - jb.tile0) * R;
+    const int row0 = (t - jb.tile0) * R, rmax = static_cast<int>(jb.n - 1);
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
-      int64_t r = row0 + gq + 8 * hh;
-      if (r >= jb.n) r = jb.n - 1;  // a valid row; results past n are never stored
-      c[hh] = jb.codes + r * row_bytes + kw * UB + lane_c;
-      sc[hh] = jb.scales + r * nG + kw * SPU + lane_s;
-      if constexpr (ASYM) mn[hh] = jb.mins + r * nG + kw * SPU + lane_s;
+      // a valid row; results past n are never stored
+      const int r = min(row0 + gq + 8 * hh, rmax);
+      c[hh] = jb.codes + static_cast<int64_t>(r) * row_bytes + (kw * UB + lane_c);
+      const int64_t so = static_cast<int64_t>(r) * nG + (kw * SPU + lane_s);
+      sc[hh] = jb.scales + so;
+      if constexpr (ASYM) mn[hh] = jb.mins + so;
     }
   };
   // fetch cursor: the next unit to load into registers
-  int64_t fi = 0;
+  int fi = 0;
   int fleft = 0;
   const uint8_t* cp[2] = {nullptr, nullptr};
   const uint16_t* sp[2] = {nullptr, nullptr};
   const uint16_t* mp[2] = {nullptr, nullptr};
-  auto set_tile = [&](int64_t i) {
+  auto set_tile = [&](int i) {
     if (i >= my_tiles) return;
     tile_ptrs(i, cp, sp, mp);
     fleft = upw;
@@ -408,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
   const uint32_t z0 = xs_a + zoff + 64u, z1 = xs_a + zoff;  // zero blocks for h = 0, 1
   uint32_t xl = 0, bl = 0;
   int cleft = 0;
-  int64_t ci = 0;
+  int ci = 0;
   auto start_tile = [&]() {
     xl = xs_a + static_cast<uint32_t>((kw * 8 + gq) * 64);
     bl = sbf_a + static_cast<uint32_t>((kw * 8 + 2 * tq) * 8);
@@ -422,12 +429,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const uint32_t ba = h ? (act1 ? xl : z1) : (act0 ? xl : z0);
-      uint32_t hs0[2] = {0u, 0u}, hs1[2] = {0u, 0u};
+      uint32_t hs0[4] = {0u, 0u, 0u, 0u}, hs1[4] = {0u, 0u, 0u, 0u};
       if constexpr (Q == 3) {
-        hs0[0] = spread_high(rg.w[0][h][2], 0);
-        hs0[1] = spread_high(rg.w[0][h][2], 1);
-        hs1[0] = spread_high(rg.w[1][h][2], 0);
-        hs1[1] = spread_high(rg.w[1][h][2], 1);
+#pragma unroll
+        for (int wi = 0; wi < 2; ++wi) {
+          hs0[wi] = high_halves(rg.w[0][h][2], wi);
+          hs1[wi] = high_halves(rg.w[1][h][2], wi);
+          hs0[2 + wi] = hs0[wi] >> 3;
+          hs1[2 + wi] = hs1[wi] >> 3;
+        }
       }
 #pragma unroll
       for (int jm = 0; jm < NP / 2; jm += 2) {
@@ -479,7 +489,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
   // End of the compute cursor's tile i: the warp's two row partials (rows
   // gq and gq + 8, summed over the quad) go straight to y (KW = 1) or to the
   // warp's slot of the partial array (KW > 1), summed after the last unit.
-  auto tile_end = [&](int64_t i) {
+  auto tile_end = [&](int i) {
     float v[2];
 #pragma unroll
     for (int hh = 0; hh < 2; ++hh) {
@@ -491,11 +501,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
     }
     if (tq != 0) return;
     if (KW == 1) {
-      const int64_t t = tfirst + i * tstride;
+      const int t = tfirst + i * tstride;
       int j = 0;
       while (j + 1 < a.njobs && t >= a.job[j + 1].tile0) ++j;
       const StreamJob& jb = a.job[j];
-      const int64_t row0 = (t - jb.tile0) * R;
+      const int64_t row0 = static_cast<int64_t>(t - jb.tile0) * R;
 #pragma unroll
       for (int hh = 0; hh < 2; ++hh) {
         const int64_t r = row0 + gq + 8 * hh;
@@ -503,7 +513,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
       }
       return;
     }
-    float* pb = part + ((static_cast<size_t>(grp) * a.rounds + i) * KW + kw) * R;
+    // the CTA's j-th tile, j = i * ngrp + grp, is tile j * grid + blockIdx.x
+    float* pb = part + (static_cast<size_t>(i * ngrp + grp) * KW + kw) * R;
     pb[gq] = v[0];
     pb[gq + 8] = v[1];
   };
@@ -540,23 +551,39 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
     }
   }
   if (KW == 1) return;
-  // ---- the sums of the tiles' KW partials, in warp order (warps without
-  // units left no partial) ----
-  __syncthreads();
-  const int kwn = KW < nunits ? KW : nunits;
-  const int per_grp = a.rounds * R;
-  for (int idx = threadIdx.x; idx < ngrp * per_grp; idx += kThreads) {
-    const int g = idx / per_grp, i = (idx / R) % a.rounds, row = idx % R;
-    const int64_t t = (static_cast<int64_t>(i) * ngrp + g) * gridDim.x + blockIdx.x;
-    if (t >= a.ntiles) continue;
-    int j = 0;
-    while (j + 1 < a.njobs && t >= a.job[j + 1].tile0) ++j;
-    const int64_t r = (t - a.job[j].tile0) * R + row;
-    if (r >= a.job[j].n) continue;
-    const float* pb = part + (static_cast<size_t>(g) * a.rounds + i) * KW * R + row;
-    float sum = 0.f;
-    for (int c = 0; c < kwn; ++c) sum += pb[c * R];
-    a.job[j].y[r] = sum;
+  // ---- the sums of the tiles' KW partials, in warp order (the host keeps KW
+  // within the units, so every warp left one); where an output goes is worked
+  // out before the barrier ----
+  const int outs = a.rounds * ngrp * R;
+  bool met = false;
+  for (int idx = threadIdx.x; idx < outs || !met; idx += kThreads) {
+    const int t = (idx / R) * grid + static_cast<int>(blockIdx.x);
+    float* y = nullptr;
+    if (idx < outs && t < a.ntiles) {
+      int j = 0;
+      while (j + 1 < a.njobs && t >= a.job[j + 1].tile0) ++j;
+      const int64_t r = static_cast<int64_t>(t - a.job[j].tile0) * R + idx % R;
+      if (r < a.job[j].n) y = a.job[j].y + r;
+    }
+    if (!met) {
+      __syncthreads();
+      met = true;
+    }
+    if (y == nullptr) continue;
+    const float* pb = part + static_cast<size_t>(idx / R) * KW * R + idx % R;
+    float sum = pb[0] + pb[R];
+    auto more = [&](auto n_tag) {
+      constexpr int N = decltype(n_tag)::value;
+      float v[N];
+#pragma unroll
+      for (int c = 2; c < N; ++c) v[c] = pb[c * R];
+#pragma unroll
+      for (int c = 2; c < N; ++c) sum += v[c];
+    };
+    if (lgkw == 2) more(std::integral_constant<int, 4>{});
+    if (lgkw == 3) more(std::integral_constant<int, 8>{});
+    if (lgkw == 4) more(std::integral_constant<int, 16>{});
+    *y = sum;
   }
 }
 
@@ -599,10 +626,11 @@ cudaError_t launch_q(const sss_qtensor_t* const* ts, StreamArgs& a, bool pdl,
                      cudaStream_t stream) {
   int64_t tiles = 0;
   for (int j = 0; j < a.njobs; ++j) {
-    a.job[j].tile0 = tiles;
+    a.job[j].tile0 = static_cast<int>(tiles);
     tiles += (ts[j]->n + 15) / 16;
   }
-  a.ntiles = tiles;
+  if (tiles > (int64_t{1} << 30)) return cudaErrorNotSupported;  // (four matrices of 2^31 rows: 2^29)
+  a.ntiles = static_cast<int>(tiles);
   // One CTA per SM (fewer when there are fewer tiles); CTA c takes tiles
   // c, c + grid, ...  Warps per tile: the power of two that minimises the
   // busiest warp's units (rounds of that CTA's tiles x units per warp per
