@@ -110,21 +110,31 @@ __device__ __forceinline__ void rotl64(uint32_t& lo, uint32_t& hi, int n) {
   hi = __funnelshift_l(a, b, n & 31);
 }
 
-// Pack the run's 32 codes and store them.  u[4j + e] is element
-// 4 * ((j + r) & 7) + e of the run (the chunk order the lane read in);
-// lg = the run's index within its group.
+// sum of kMagic's bits times 2^(B e), e = 0 .. n - 1, modulo 2^32
+constexpr uint32_t magic_sum(int B, int n) {
+  uint32_t v = 0;
+  for (int e = 0; e < n; ++e) v += 0x4B400000u << (B * e);
+  return v;
+}
+
+// Pack the run's 32 codes and store them.  t[4j + e] is kMagic + the code of
+// element 4 * ((j + r) & 7) + e of the run (the chunk order the lane read in);
+// lg = the run's index within its group.  A word's codes are summed with their
+// floats' bits as they are, one shift-and-add each, and the known sum of the
+// magic bits is taken off once.
 template <int Q, int G>
 __device__ __forceinline__ void store_run(uint8_t* __restrict__ codes, int64_t grp, int lg, int r,
-                                          const int (&u)[32]) {
+                                          const float (&t)[32]) {
+  auto bits = [&](int e) { return static_cast<uint32_t>(__float_as_int(t[e])); };
   if constexpr (Q == 4) {
     // chunk c's four nibbles belong at bits 16c..16c+15: pack by slot, then
     // rotate the 128-bit value left by 16r
     uint32_t P[4];
 #pragma unroll
     for (int wd = 0; wd < 4; ++wd) {
-      uint32_t v = 0;
+      uint32_t v = 0u - magic_sum(4, 8);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v |= static_cast<uint32_t>(u[8 * wd + e]) << (4 * e);
+      for (int e = 0; e < 8; ++e) v += bits(8 * wd + e) << (4 * e);
       P[wd] = v;
     }
     if (r & 1) {
@@ -140,23 +150,33 @@ __device__ __forceinline__ void store_run(uint8_t* __restrict__ codes, int64_t g
     const uint4 out = make_uint4(w2 ? t2 : t0, w2 ? t3 : t1, w2 ? t0 : t2, w2 ? t1 : t3);
     reinterpret_cast<uint4*>(codes + grp * (G / 2))[lg] = out;
   } else if constexpr (Q == 2) {
-    uint32_t lo = 0, hi = 0;
+    uint32_t lo = 0u - magic_sum(2, 16), hi = lo;
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
-      lo |= static_cast<uint32_t>(u[e]) << (2 * e);
-      hi |= static_cast<uint32_t>(u[16 + e]) << (2 * e);
+      lo += bits(e) << (2 * e);
+      hi += bits(16 + e) << (2 * e);
     }
     rotl64(lo, hi, 8 * r);
     reinterpret_cast<uint2*>(codes + grp * (G / 4))[lg] = make_uint2(lo, hi);
   } else {  // low 2-bit plane (q=2 layout), then the high-bit plane
-    uint32_t l0 = 0, l1 = 0, hi = 0;
+    // sums of the codes and of their high bits h (u = lo + 4h) at two bits each;
+    // the first less four times the second is the low plane, and the second
+    // closes up to the high one
+    uint32_t l[2], hp[2];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      l0 |= static_cast<uint32_t>(u[e] & 3) << (2 * e);
-      l1 |= static_cast<uint32_t>(u[16 + e] & 3) << (2 * e);
+    for (int k = 0; k < 2; ++k) {
+      uint32_t v = 0u - magic_sum(2, 16), h = (bits(16 * k) & 4u) >> 2;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) v += bits(16 * k + e) << (2 * e);
+#pragma unroll
+      for (int e = 1; e < 16; ++e) h += (bits(16 * k + e) & 4u) << (2 * e - 2);
+      l[k] = v - (h << 2);
+      h = (h | (h >> 1)) & 0x33333333u;
+      h = (h | (h >> 2)) & 0x0F0F0F0Fu;
+      h = (h | (h >> 4)) & 0x00FF00FFu;
+      hp[k] = (h | (h >> 8)) & 0xFFFFu;
     }
-#pragma unroll
-    for (int e = 0; e < 32; ++e) hi |= static_cast<uint32_t>(u[e] >> 2) << e;
+    uint32_t l0 = l[0], l1 = l[1], hi = hp[0] | (hp[1] << 16);
     rotl64(l0, l1, 8 * r);
     hi = __funnelshift_l(hi, hi, 4 * r);
     uint32_t* base = reinterpret_cast<uint32_t*>(codes + grp * (3 * G / 8));
@@ -166,7 +186,7 @@ __device__ __forceinline__ void store_run(uint8_t* __restrict__ codes, int64_t g
   }
 }
 
-// Quantize one run of 32 weights (x[4j + e] = element 4*((j + r) & 7) + e,
+// Quantize one run of 32 weights (x2[p] packs x[2p], x[2p + 1]; x[4j + e] = element 4*((j + r) & 7) + e,
 // run index gr in the flat weight array) together with the other runs of
 // its group (the L = G/32 consecutive lanes of the warp): group max / min,
 // scale, codes, packing, scale / min / clip-count stores.  Every lane of
@@ -174,7 +194,7 @@ __device__ __forceinline__ void store_run(uint8_t* __restrict__ codes, int64_t g
 // re-reads x[e] as it was passed in (the rare exact-tie decisions use it,
 // so x need not stay live in registers).
 template <int Q, int GRID, int G, bool STATS, class Wat>
-__device__ __forceinline__ void quantize_run(float (&x)[32], Wat wat, int r, bool valid, int64_t gr,
+__device__ __forceinline__ void quantize_run(uint64_t (&x2)[16], Wat wat, int r, bool valid, int64_t gr,
                                              uint8_t* __restrict__ codes,
                                              uint16_t* __restrict__ scales,
                                              uint16_t* __restrict__ mins,
@@ -188,11 +208,18 @@ __device__ __forceinline__ void quantize_run(float (&x)[32], Wat wat, int r, boo
   const int lg = static_cast<int>(gr % L);
   // max with NaN propagation: a NaN anywhere makes mx NaN, an infinity
   // makes mx or mn infinite, so the run is non-finite iff they are
-  float mx = x[0], mn = x[0];
+  float mx, mn;
+  {
+    float x0, x1;
+    unpack2(x2[0], x0, x1);
+    mx = mn = x0;
 #pragma unroll
-  for (int e = 0; e < 32; ++e) {
-    asm("max.NaN.f32 %0, %0, %1;" : "+f"(mx) : "f"(x[e]));
-    mn = fminf(mn, x[e]);
+    for (int p = 0; p < 16; ++p) {
+      unpack2(x2[p], x0, x1);
+      asm("max.NaN.f32 %0, %0, %1;" : "+f"(mx) : "f"(x0));
+      asm("max.NaN.f32 %0, %0, %1;" : "+f"(mx) : "f"(x1));
+      mn = fminf(mn, fminf(x0, x1));
+    }
   }
   unsigned bad = (is_nonfinite(mx) || is_nonfinite(mn)) ? 1u : 0u;
 #pragma unroll
@@ -202,7 +229,8 @@ __device__ __forceinline__ void quantize_run(float (&x)[32], Wat wat, int r, boo
     bad |= __shfl_xor_sync(0xffffffffu, bad, o);
   }
   unsigned flags = bad ? SSS_FLAG_NONFINITE : 0u;
-  int u[32];
+  float u[32];  // kMagic + code
+  constexpr float TOP = kMagic + static_cast<float>(UMAX);
   int n_self = 0, n_other = 0;
   uint16_t s16, m16 = 0;
   if constexpr (GRID != SSS_GRID_ASYM) {
@@ -217,7 +245,7 @@ __device__ __forceinline__ void quantize_run(float (&x)[32], Wat wat, int r, boo
     const float s = zero ? 0.f : gamma * alpha;
     if (zero) {
 #pragma unroll
-      for (int e = 0; e < 32; ++e) u[e] = HALF;
+      for (int e = 0; e < 32; ++e) u[e] = kMagic + static_cast<float>(HALF);
     } else {
       float ss = s, sig = 1.f;
       // alpha is an exact power-of-two scaling of M unless it is
@@ -228,22 +256,26 @@ __device__ __forceinline__ void quantize_run(float (&x)[32], Wat wat, int r, boo
         sig = (M < 1.f) ? 0x1p+64f : 0x1p-64f;
         ss = __fmul_rn(s, sig);
 #pragma unroll
-        for (int e = 0; e < 32; ++e) x[e] = __fmul_rn(x[e], sig);
+        for (int p = 0; p < 16; ++p) {
+          float x0, x1;
+          unpack2(x2[p], x0, x1);
+          x2[p] = pack2(__fmul_rn(x0, sig), __fmul_rn(x1, sig));
+        }
       }
       const float rc = __frcp_rn(ss);
       // c_pre + 2^(q-1); w * 1 is w, so the re-read matches x in both cases
-      codes_of<OFF>(x, ss, rc, u, [&](int e) { return __fmul_rn(wat(e), sig); });
+      codes_of<OFF>(x2, ss, rc, u, [&](int e) { return __fmul_rn(wat(e), sig); });
 #pragma unroll
       for (int e = 0; e < 32; ++e) {
         if constexpr (STATS) {
-          n_self += (u[e] == 2 * HALF);  // c_pre == +2^(q-1): in C_gamma
-          n_other += (u[e] == 0);        // c_pre == -2^(q-1): in C_-gamma
+          n_self += (u[e] == kMagic + static_cast<float>(2 * HALF));  // c_pre == +2^(q-1): in C_gamma
+          n_other += (u[e] == kMagic);  // c_pre == -2^(q-1): in C_-gamma
         }
-        u[e] = min(u[e], UMAX);
+        u[e] = fminf(u[e], TOP);
       }
       if (lo_clip) {
 #pragma unroll
-        for (int e = 0; e < 32; ++e) u[e] = max(u[e], 0);
+        for (int e = 0; e < 32; ++e) u[e] = fmaxf(u[e], kMagic);
       }
     }
     s16 = __half_as_ushort(__float2half_rn(s));
@@ -263,7 +295,7 @@ __device__ __forceinline__ void quantize_run(float (&x)[32], Wat wat, int r, boo
     }
     if (zero) {
 #pragma unroll
-      for (int e = 0; e < 32; ++e) u[e] = 0;
+      for (int e = 0; e < 32; ++e) u[e] = kMagic;
     } else {
       float ss = s, sig = 1.f;
       if (s < 0x1p-96f || s > 0x1p+96f) {
@@ -272,16 +304,23 @@ __device__ __forceinline__ void quantize_run(float (&x)[32], Wat wat, int r, boo
       }
       const float rc = __frcp_rn(ss);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) {
-        x[e] = __fsub_rn(x[e], mn);  // fl32(w - min) >= 0
-        if (sig != 1.f) x[e] = __fmul_rn(x[e], sig);
+      for (int p = 0; p < 16; ++p) {
+        float x0, x1;
+        unpack2(x2[p], x0, x1);
+        x0 = __fsub_rn(x0, mn);  // fl32(w - min) >= 0
+        x1 = __fsub_rn(x1, mn);
+        if (sig != 1.f) {
+          x0 = __fmul_rn(x0, sig);
+          x1 = __fmul_rn(x1, sig);
+        }
+        x2[p] = pack2(x0, x1);
       }
-      codes_of<0>(x, ss, rc, u, [&](int e) {
+      codes_of<0>(x2, ss, rc, u, [&](int e) {
         const float d = __fsub_rn(wat(e), mn);
         return sig != 1.f ? __fmul_rn(d, sig) : d;
       });
 #pragma unroll
-      for (int e = 0; e < 32; ++e) u[e] = min(u[e], UMAX);
+      for (int e = 0; e < 32; ++e) u[e] = fminf(u[e], TOP);
     }
     s16 = __half_as_ushort(__float2half_rn(s));  // inf when the step overflowed
     m16 = __half_as_ushort(__float2half_rn(mn));
@@ -371,16 +410,15 @@ __global__ void __launch_bounds__(kQThreads, 1)
       const int64_t w0 = (blockIdx.x + i * gridDim.x) * static_cast<int64_t>(kQChunk);
       const int64_t nrun = (nweights - w0 < kQChunk ? nweights - w0 : kQChunk) / 32;
       const bool valid = sl < nrun;
-      float x[32];
+      uint64_t x[16];
       const uint32_t run_a = q_su32(smem + s * kQChunk * 4 + sl * 128);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        x[2 * j] = x[2 * j + 1] = 0ull;
         if (valid)
-          asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
-                       : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+          asm volatile("ld.shared.v2.b64 {%0,%1}, [%2];"
+                       : "=l"(x[2 * j]), "=l"(x[2 * j + 1])
                        : "r"(run_a + 16u * static_cast<uint32_t>((j + r) & 7)));
-        x[4 * j] = v.x; x[4 * j + 1] = v.y; x[4 * j + 2] = v.z; x[4 * j + 3] = v.w;
       }
       // the stage is released after the run is quantized: the rare exact
       // tie decisions re-read their weights from it
@@ -505,25 +543,11 @@ constexpr int kRGroups = 3;   // divides the stages: each group has its own (see
 constexpr int kRThreads = 32 + 128 * kRGroups;
 static_assert(kQStages % kRGroups == 0, "a group waits for every phase of its stages");
 
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // the butterflies between pairs p and p + D (a multiple of pairs apart)
 template <int D>
 __device__ __forceinline__ void stage2(uint64_t (&v)[32], uint64_t neg1) {
@@ -743,7 +767,7 @@ __global__ void __launch_bounds__(kRThreads, 1)
     for (int sl = t; sl < kQChunk / 32; sl += 128) {
       const bool valid = 32 * sl < nv;
       const uint32_t run_a = base + 128u * static_cast<uint32_t>(sl);
-      float x[32];
+      uint64_t x[16];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -751,8 +775,10 @@ __global__ void __launch_bounds__(kRThreads, 1)
           asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
                        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                        : "r"(run_a + 16u * static_cast<uint32_t>((j + r) & 7)));
-        x[4 * j] = __fmul_rn(v.x, norm); x[4 * j + 1] = __fmul_rn(v.y, norm);
-        x[4 * j + 2] = __fmul_rn(v.z, norm); x[4 * j + 3] = __fmul_rn(v.w, norm);
+        // (scalar products: a packed one could be contracted into the min-max
+        // grid's subtraction)
+        x[2 * j] = pack2(__fmul_rn(v.x, norm), __fmul_rn(v.y, norm));
+        x[2 * j + 1] = pack2(__fmul_rn(v.z, norm), __fmul_rn(v.w, norm));
       }
       quantize_run<Q, GRID, G, STATS>(
           x,

@@ -55,27 +55,50 @@ __device__ __forceinline__ int code_of(float w, float s, float r) {
   return u;
 }
 
-// The same for N weights at once (the same codes as N calls of code_of):
-// every weight's rounding in one straight line, so the N chains
-// interleave, and a single branch, taken only when some weight lies within
-// 2^-18 of a half-integer, into the exact side decisions.  That branch
-// takes weight e from wat(e), which must return the value w[e] held, so
-// that w need not stay in registers past the straight line.
+// two fp32 values as the packed operand of the two-wide fp32 instructions
+// (each half rounds as the scalar instruction)
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// The same for 2N weights at once (w[p] holds weights 2p and 2p + 1; the same
+// codes as 2N calls of code_of): every weight's rounding in one straight line,
+// two weights to an instruction, and a single branch, taken only when some
+// weight lies within 2^-18 of a half-integer (w*r - c is at most 1/2 in
+// magnitude), into the exact side decisions.  That branch takes weight e from
+// wat(e), which must return the value held in w, so that w need not stay in
+// registers past the straight line.  t[e] is returned as the float kMagic + u,
+// whose low bits are the code: it is clamped and packed as it is.
 template <int OFF, int N, class Wat>
-__device__ __forceinline__ void codes_of(const float (&w)[N], float s, float r, int (&u)[N],
-                                         Wat wat) {
+__device__ __forceinline__ void codes_of(const uint64_t (&w)[N], float s, float r,
+                                         float (&t)[2 * N], Wat wat) {
   constexpr float MAGIC = kMagic + static_cast<float>(OFF);
-  float near = 1.f;
+  const uint64_t r2 = pack2(r, r), m2 = pack2(MAGIC, MAGIC), neg1 = pack2(-1.f, -1.f);
+  float near = 0.f;
 #pragma unroll
-  for (int e = 0; e < N; ++e) {
-    const float t = __fmaf_rn(w[e], r, MAGIC);
-    u[e] = __float_as_int(t) - __float_as_int(kMagic);
-    const float dd = __fmaf_rn(w[e], r, __fsub_rn(MAGIC, t));
-    near = fminf(near, fabsf(__fsub_rn(fabsf(dd), 0.5f)));
+  for (int p = 0; p < N; ++p) {
+    const uint64_t t2 = fma2(w[p], r2, m2);
+    float d0, d1;
+    unpack2(fma2(w[p], r2, fma2(neg1, t2, m2)), d0, d1);  // w*r - c; MAGIC - t = -c exactly
+    near = fmaxf(near, fmaxf(fabsf(d0), fabsf(d1)));
+    unpack2(t2, t[2 * p], t[2 * p + 1]);
   }
-  if (near <= 0x1p-18f) {  // unrolled: u stays in registers
+  if (near >= 0.5f - 0x1p-18f) {  // unrolled: t stays in registers
 #pragma unroll
-    for (int e = 0; e < N; ++e) u[e] = fix_tie<OFF>(wat(e), s, r, u[e]);
+    for (int e = 0; e < 2 * N; ++e) {
+      const int u = __float_as_int(t[e]) - __float_as_int(kMagic);
+      t[e] = __int_as_float(__float_as_int(kMagic) + fix_tie<OFF>(wat(e), s, r, u));
+    }
   }
 }
 
