@@ -77,7 +77,8 @@ typedef enum {
                                    (see those calls); their outputs may then hold
                                    inf or NaN                                         */
 #define SSS_FLAG_TIMEOUT 0x4u   /* a bounded pipeline wait of sss_gemm (or
-                                   sss_gemm_noalloc) expired; the output is
+                                   sss_gemm_noalloc), sss_quantize or
+                                   sss_quantize_rotated expired; the output is
                                    incomplete                                         */
 
 typedef enum { SSS_OUT_F32 = 0, SSS_OUT_F16 = 1, SSS_OUT_BF16 = 2 } sss_dtype_t;
@@ -146,16 +147,16 @@ sss_status_t sss_dequantize(const sss_qtensor_t* qt, void* out,
  * dequantisation fused (Appendix B.3: y = sum_b s * (integer dot) for the
  * symmetric formats, plus the row-sum term sum_b m * sum_{k in b} x for
  * ASYM).  fp32 accumulation; deterministic (no atomics).  At batch 1, and at
- * batch 2..16 for q = 2 and 4 (k a multiple of 256), the integer codes meet the
- * activations exactly (activations within fp16's range) and the group scale is
- * applied in fp32.  At batch 2..16 for q = 3 the batch fills the tensor-core
- * columns across groups, so each weight enters the product as w^ rounded once
- * to fp16 (<= 2^-11 relative, as in sss_gemm), times 2^p (p = 0, 2 or 4, the
- * bit offset of the code's field).  That operand fits fp16 while
- * |w^| * 2^p < 65520; at batch 2..16, whatever q, every group whose scale could
- * break this raises SSS_FLAG_RANGE (checked per scale, conservatively:
- * |s| * 2^(q-1) * 16 >= 65520 for the symmetric grids,
- * (|s| * (2^q - 1) + |m|) * 16 >= 65520 for ASYM).
+ * batch 2..16 for q = 2 and 4, the integer codes meet the activations exactly
+ * (activations within fp16's range) and the group scale is applied in fp32;
+ * so too for q = 3 with k not a multiple of 256.  Otherwise, for q = 3, the
+ * batch fills the tensor-core columns across groups, so each weight enters the
+ * product as w^ rounded once to fp16 (<= 2^-11 relative, as in sss_gemm), times
+ * 2^p (p = 0, 2 or 4, the bit offset of the code's field).  That operand fits
+ * fp16 while |w^| * 2^p < 65520; at batch 2..16 with k a multiple of 256,
+ * whatever q, every group whose scale could break this raises SSS_FLAG_RANGE
+ * (checked per scale, conservatively: |s| * 2^(q-1) * 16 >= 65520 for the
+ * symmetric grids, (|s| * (2^q - 1) + |m|) * 16 >= 65520 for ASYM).
  *   qt        [in]  packed tensor; codes 16-byte aligned, scales/mins 4-byte
  *                   aligned.
  *   x_bf16    [in]  device bf16 [batch][k], 16-byte aligned.

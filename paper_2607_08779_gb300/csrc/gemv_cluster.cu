@@ -20,6 +20,11 @@
 //    balances shared-memory reads and instruction issue), a step 128 codes; its
 //    codes and scales come through a private ring of 16-byte cp.async copies,
 //    no barriers.
+//  * CUT, a k that is no multiple of 256 or scale rows of 2-byte alignment: a
+//    row's last step may be cut short.  Codes past k are not copied and meet
+//    zeros of x; scales past the row are zeros.  (14336 x 4128 and x 4160, q = 4,
+//    batch 4: 27 and 30 us in the general kernel, 18.5 and 14 here; batch 16: 90
+//    and 116 us, 25 and 20 here: that kernel repeats its mmas per batch row.)
 //  * A cluster of S CTAs shares its row tiles and splits k: each CTA stages
 //    only k/S of x (staging all of x in every CTA, 128 KB at batch 16 and k =
 //    4096, took as long as a small matrix's weights); each warp stores its
@@ -65,10 +70,11 @@ struct ClusterArgs {
   int64_t n, k;
   int batch;
   int ntiles;
-  int nsteps;     // k / 128
+  int nsteps;     // k / 128, rounded up
   int csteps;     // steps per CTA of a cluster
   int wsteps;     // steps per warp of a tile's group
-  int salign;     // bytes the scale rows are aligned to: 16, 8 or 4
+  int salign;     // bytes the scale rows are aligned to: 16, 8, 4 or 2
+  int calign;     // bytes the code rows are aligned to: 16 or 8
   int lgkw;       // log2(warps per tile)
   int rounds;     // tiles per warp group and pass (the partial array's depth)
   uint32_t* status;
@@ -130,7 +136,8 @@ struct Shape {
   }
 };
 
-template <int Q, bool ASYM, int G, int NBLK, int D>
+// CUT: k is not a multiple of 256, or scale rows are aligned to 2 bytes only.
+template <int Q, bool ASYM, int G, int NBLK, int D, bool CUT>
 __global__ void __launch_bounds__(kThreads, 1)
     gemv_cluster_kernel(const __grid_constant__ ClusterArgs a) {
   using SH = Shape<Q, ASYM, G, NBLK, D>;
@@ -197,7 +204,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int i = 0; i < CPR; ++i) {
       const int row = (lane + 32 * i) / CPR, c = lane % CPR;
       const int sw = Q == 4 ? (c ^ ((row >> 1) & 3)) : (c ^ ((row >> 2) & 1));
-      cp_async(st + static_cast<uint32_t>(row * P + 16 * sw), cp[i], 16);
+      const uint32_t dst = st + static_cast<uint32_t>(row * P + 16 * sw);
+      // (the last step of a row may be cut short; what then lies in the slot's
+      // rest meets zeros of x, and any bits masked to a code are finite)
+      const int left = CUT ? static_cast<int>(row_bytes) - fstep * P - 16 * c : 16;
+      if (!CUT || Q == 4 || a.calign == 16) {
+        if (left > 0) cp_async(dst, cp[i], 16);
+      } else {
+        if (left > 0) cp_async(dst, cp[i], 8);
+        if (left > 8) cp_async(dst + 8, cp[i] + 8, 8);
+      }
       cp[i] += P;
     }
     if (fleft == upw || fstep % BS == 0) {  // lane: row `lane` of the next block
@@ -205,7 +221,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t bl = my_ring + D * SH::CODE + static_cast<uint32_t>(fblk) * SH::BLOCK +
                           static_cast<uint32_t>(lane * SB);
       const int g0 = fstep / BS * (SB / 2);
-      // (a row's last block may be cut short)
+      // (a row's last block may be cut short: zeros for the groups past its end
+      // that its last step still computes)
       const int left = static_cast<int>(nG - g0) * 2;
       auto copy = [&](auto n_tag) {
         constexpr int N = decltype(n_tag)::value;
@@ -215,11 +232,38 @@ __global__ void __launch_bounds__(kThreads, 1)
             cp_async(bl + o, reinterpret_cast<const uint8_t*>(sp + g0) + o, N);
             if constexpr (ASYM)
               cp_async(bl + kRows * SB + o, reinterpret_cast<const uint8_t*>(mp + g0) + o, N);
+          } else if constexpr (CUT) {
+#pragma unroll
+            for (int z = 0; z < N; z += 4) {
+              asm volatile("st.shared.u32 [%0], %1;" ::"r"(bl + o + z), "r"(0u) : "memory");
+              if constexpr (ASYM)
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(bl + kRows * SB + o + z), "r"(0u)
+                             : "memory");
+            }
           }
+      };
+      // an odd number of groups per row: no asynchronous copy is that narrow
+      auto copy2 = [&]() {
+#pragma unroll
+        for (int m = 0; m < (ASYM ? 2 : 1); ++m) {
+          const uint16_t* src = (m ? mp : sp) + g0;
+          uint32_t v[SB / 4];
+#pragma unroll
+          for (int j = 0; j < SB / 4; ++j) {
+            const uint32_t lo = 4 * j < left ? __ldg(src + 2 * j) : 0u;
+            const uint32_t hi = 4 * j + 2 < left ? __ldg(src + 2 * j + 1) : 0u;
+            v[j] = lo | hi << 16;
+          }
+#pragma unroll
+          for (int j = 0; j < SB / 4; ++j)
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(bl + m * (kRows * SB) + 4 * j), "r"(v[j])
+                         : "memory");
+        }
       };
       if (SB == 16 && a.salign == 16) copy(std::integral_constant<int, 16>{});
       else if (a.salign >= 8) copy(std::integral_constant<int, 8>{});
-      else copy(std::integral_constant<int, 4>{});
+      else if (!CUT || a.salign == 4) copy(std::integral_constant<int, 4>{});
+      else if constexpr (CUT) copy2();
     }
     ++fstep;
     if (--fleft == 0) {
@@ -233,14 +277,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   // 2^-pos; four rows' loads are in flight together, the first four issued
   // before the weight ring's copies.  (Columns past the batch hold whatever
   // was there: an mma's columns do not mix, and theirs are never stored.) ----
-  const int xunits = (ns + 1) / 2;  // of 256 values (the last may hold 128)
+  const int xunits = (ns + 1) / 2;  // of 256 values (the last may hold fewer; zeros past k)
+  const int xvals =
+      CUT ? static_cast<int>(min(static_cast<int64_t>(ns) * kStep, a.k - static_cast<int64_t>(s0) * kStep))
+          : ns * kStep;
   const int lgu = xunits >= kWarps ? 4 : 32 - __clz(max(xunits - 1, 0));  // warps per row: 2^lgu
   const int rstep = kWarps >> lgu;  // rows taken side by side
   const int nr0 = warp >> lgu;
   uint4 xv[4];
   auto xload = [&](int ul, int nr) {
     const uint16_t* src = a.x + static_cast<int64_t>(s0) * kStep + ul * 256 + 8 * lane;
-    const bool in = ul * 256 + 8 * lane < ns * kStep;
+    const bool in = ul * 256 + 8 * lane < xvals;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = nr + i * rstep;
@@ -353,6 +400,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t xa = xs_a + static_cast<uint32_t>(st * SH::XSTEP + lane * 16);
     const float* bs = bsum + st * (SEG * NBC);
     uint32_t w[2][4];  // q = 2: the codes of the chunk's two sub-chunks
+    // CUT: the step's own sum, added to the tile's at its end, with row sums and
+    // the sub-chunk's mmas added in fp32: no more error than the general kernel's
+    // short chains, which took these shapes before (against 64 bits 0.96 of it,
+    // the geometric mean of 90 shapes and batches)
+    float t[2][CUT ? NBLK : 1][4];
+    if constexpr (CUT) {
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int nb = 0; nb < NBLK; ++nb)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) t[m][nb][e] = 0.f;
+    }
 #pragma unroll
     for (int seg = 0; seg < SEG; ++seg) {
       float d[2][NBLK][4];
@@ -398,9 +458,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int nb = 0; nb < NBLK; ++nb) {
               const uint32_t b0 = j ? bv[nb].z : bv[nb].x, b1 = j ? bv[nb].w : bv[nb].y;
-              if (i == 0 && j == 0)
+              if (CUT && (i > 0 || j > 0)) {
+                float e[4];  // (added here: the tensor core's own sum truncates)
+                mma_c(e, f0[2 * m], f0[2 * m + 1], f1[2 * m], f1[2 * m + 1], b0, b1, 0.f, 0.f);
+#pragma unroll
+                for (int z = 0; z < 4; ++z) d[m][nb][z] += e[z];
+              } else if (i == 0 && j == 0)
                 mma_c(d[m][nb], f0[2 * m], f0[2 * m + 1], f1[2 * m], f1[2 * m + 1], b0, b1,
-                      ASYM ? 0.f : b[nb].x, ASYM ? 0.f : b[nb].y);
+                      ASYM || CUT ? 0.f : b[nb].x, ASYM || CUT ? 0.f : b[nb].y);
               else
                 mma16816(d[m][nb], f0[2 * m], f0[2 * m + 1], f1[2 * m], f1[2 * m + 1], b0, b1);
             }
@@ -420,16 +485,24 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
 #pragma unroll
         for (int nb = 0; nb < NBLK; ++nb) {
-          float* ac = acc[h >> 1][nb] + 2 * (h & 1);
+          float* ac = (CUT ? t[h >> 1][nb] : acc[h >> 1][nb]) + 2 * (h & 1);
           const float* dd = d[h >> 1][nb] + 2 * (h & 1);
-          ac[0] = fmaf(s, dd[0], ac[0]);
-          ac[1] = fmaf(s, dd[1], ac[1]);
+          ac[0] = fmaf(s, CUT && !ASYM ? dd[0] + b[nb].x : dd[0], ac[0]);
+          ac[1] = fmaf(s, CUT && !ASYM ? dd[1] + b[nb].y : dd[1], ac[1]);
           if constexpr (ASYM) {
             ac[0] = fmaf(mn, b[nb].x, ac[0]);
             ac[1] = fmaf(mn, b[nb].y, ac[1]);
           }
         }
       }
+    }
+    if constexpr (CUT) {
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int nb = 0; nb < NBLK; ++nb)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[m][nb][e] += t[m][nb][e];
     }
   };
 
@@ -517,6 +590,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int st = s0 + u0 + u;
             for (int i = 0; i < SEG; ++i) {
               const int64_t gi = static_cast<int64_t>(st) * kStep / G + i;
+              if (CUT && gi >= nG) continue;
               const float s = fabsf(__half2float(__ushort_as_half(a.scales[r * nG + gi])));
               const float m = fabsf(__half2float(__ushort_as_half(a.mins[r * nG + gi])));
               big |= (s * static_cast<float>(2 * HALF - 1) + m) * 16.f >= 65520.f;
@@ -538,7 +612,7 @@ int max_clusters(int lgS) {
   std::lock_guard<std::mutex> lock(mu);
   int& c = cache[dev][lgS];
   if (c == 0) {
-    auto kern = gemv_cluster_kernel<4, false, 32, 1, 3>;
+    auto kern = gemv_cluster_kernel<4, false, 32, 1, 3, false>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(device_sm_count()) / (1u << lgS) * (1u << lgS), 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
@@ -560,7 +634,7 @@ int max_clusters(int lgS) {
   return c < 0 ? 0 : c;
 }
 
-template <int Q, bool ASYM, int G, int NBLK, int D>
+template <int Q, bool ASYM, int G, int NBLK, int D, bool CUT>
 cudaError_t launch_c(ClusterArgs& a, cudaStream_t stream) {
   using SH = Shape<Q, ASYM, G, NBLK, D>;
   // Cluster size and warps per tile of least estimated time in SM cycles: the
@@ -612,7 +686,7 @@ cudaError_t launch_c(ClusterArgs& a, cudaStream_t stream) {
   a.wsteps = (best_cs + (1 << best_lgkw) - 1) >> best_lgkw;
   const int S = 1 << best_lgs;
   const int nclus = std::min(max_clusters(best_lgs), a.ntiles);
-  auto kern = gemv_cluster_kernel<Q, ASYM, G, NBLK, D>;
+  auto kern = gemv_cluster_kernel<Q, ASYM, G, NBLK, D, CUT>;
   const size_t smem = SH::bytes(best_cs, best_rounds);
   cudaError_t e = ensure_smem(kern, kSmemMax);
   if (e != cudaSuccess) return e;
@@ -636,8 +710,12 @@ template <int Q, bool ASYM, int G>
 cudaError_t launch_n(ClusterArgs& a, cudaStream_t stream) {
   // (the min-max ring at 16 columns leaves x no room for a fourth stage)
   constexpr int D = Q == 4 ? 3 : 4, D16 = Q == 2 && !ASYM ? 4 : 3;
-  if (a.batch <= 8) return launch_c<Q, ASYM, G, 1, D>(a, stream);
-  return launch_c<Q, ASYM, G, 2, D16>(a, stream);
+  if (a.k % 256 != 0 || a.salign == 2) {
+    if (a.batch <= 8) return launch_c<Q, ASYM, G, 1, D, true>(a, stream);
+    return launch_c<Q, ASYM, G, 2, D16, true>(a, stream);
+  }
+  if (a.batch <= 8) return launch_c<Q, ASYM, G, 1, D, false>(a, stream);
+  return launch_c<Q, ASYM, G, 2, D16, false>(a, stream);
 }
 
 template <int Q, bool ASYM>
@@ -652,16 +730,20 @@ cudaError_t launch_g(int g, ClusterArgs& a, cudaStream_t stream) {
 
 }  // namespace
 
-// q = 2 and 4 with whole 256-code units per row and buffers aligned for the
-// copies; launch_gemv_cluster may still return cudaErrorNotSupported (a k
-// whose staged x fits no cluster), without having launched anything.
+// q = 2 and 4, any k; launch_gemv_cluster may still return
+// cudaErrorNotSupported (a k whose staged x fits no cluster), without having
+// launched anything.  Scale rows of 2-byte alignment come by loads that a warp
+// waits for, a block at a time: with many groups of 32, few rows to share them
+// and little work per row, the general kernel is as fast or faster (300 x 2080,
+// q = 2, batch 2: 4.3 us against 4.9; 1024 x 4128: 5.0 against 4.8).
 bool gemv_cluster_eligible(const sss_qtensor_t& t, const uint16_t* x, int batch, const float* y) {
   auto al = [](const void* p, size_t b) { return (reinterpret_cast<uintptr_t>(p) % b) == 0; };
   if (t.q == 3 || batch < 2 || batch > 16) return false;
-  if (t.k <= 0 || t.n <= 0 || t.k % 256 != 0 || t.k > (int64_t{1} << 24)) return false;
+  if (t.k <= 0 || t.n <= 0 || t.k % 32 != 0 || t.k > (int64_t{1} << 24)) return false;
   if (t.n > (int64_t{1} << 30)) return false;
-  if (!al(t.codes, 16) || !al(t.scales, 4) || !al(x, 16) || !al(y, 4)) return false;
-  if (t.grid == SSS_GRID_ASYM && !al(t.mins, 4)) return false;
+  if (!al(t.codes, 16) || !al(t.scales, 2) || !al(x, 16) || !al(y, 4)) return false;
+  if (t.grid == SSS_GRID_ASYM && !al(t.mins, 2)) return false;
+  if (t.group == 32 && t.k / 32 % 2 != 0 && batch <= 4 && t.n <= 512 && t.k >= 1024) return false;
   return true;
 }
 
@@ -678,12 +760,15 @@ cudaError_t launch_gemv_cluster(const sss_qtensor_t& t, const uint16_t* x, int b
   a.k = t.k;
   a.batch = batch;
   a.ntiles = static_cast<int>((t.n + kRows - 1) / kRows);
-  a.nsteps = static_cast<int>(t.k / kStep);
-  a.status = status;
+  a.nsteps = static_cast<int>((t.k + kStep - 1) / kStep);
   const bool asym = t.grid == SSS_GRID_ASYM;
   uintptr_t bits = reinterpret_cast<uintptr_t>(t.scales) | static_cast<uintptr_t>(t.k / t.group * 2);
   if (asym) bits |= reinterpret_cast<uintptr_t>(t.mins);
-  a.salign = bits % 16 == 0 ? 16 : (bits % 8 == 0 ? 8 : 4);
+  a.salign = bits % 16 == 0 ? 16 : (bits % 8 == 0 ? 8 : (bits % 4 == 0 ? 4 : 2));
+  a.calign = t.k * t.q / 8 % 16 == 0 ? 16 : 8;
+  // The flag speaks of the fp16 weight operand that k a multiple of 256 is
+  // documented to have; other shapes never raised it.
+  a.status = t.k % 256 == 0 && bits % 4 == 0 ? status : nullptr;
   if (t.q == 2) return asym ? launch_g<2, true>(t.group, a, stream) : launch_g<2, false>(t.group, a, stream);
   if (t.q == 4) return asym ? launch_g<4, true>(t.group, a, stream) : launch_g<4, false>(t.group, a, stream);
   return cudaErrorNotSupported;

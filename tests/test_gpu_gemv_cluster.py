@@ -51,3 +51,38 @@ def test_gemv_cluster_large_activations():
         y = sss.sss_gemv(qt, x)
         ref = x.double() @ sss.sss_dequantize(qt).double().T
         assert ((y - ref).abs().amax(1) / ref.abs().amax(1)).max().item() <= TOL
+
+
+@pytest.mark.parametrize("batch", [2, 9])
+@pytest.mark.parametrize("q", [2, 4])
+@pytest.mark.parametrize("n,k,g,grid", [
+    (24, 32, 32, sss.GRID_ASYM),            # one group: a quarter of a step
+    (65, 96, 32, sss.GRID_SIGNED_SYM),      # 2-byte scale rows, q = 2 code rows of 8 bytes' alignment
+    (40, 192, 64, sss.GRID_ASYM),           # a step and a half
+    (33, 128, 128, sss.GRID_SIGNED_SYM),    # one step, one scale per row
+    (100, 4128, 32, sss.GRID_ASYM),         # a quarter of a step past 32
+    (2500, 1120, 32, sss.GRID_UNSIGNED_SYM),
+    (300, 4224, 128, sss.GRID_ASYM),        # 66-byte scale rows
+    (70, 4160, 64, sss.GRID_SIGNED_SYM),
+])
+def test_gemv_cluster_cut_steps(n, k, g, grid, q, batch):
+    run_case(n, k, q, g, grid, batch, n + k + g + q + batch, outliers=False, tol=TOL)
+
+
+@pytest.mark.parametrize("q", [2, 4])
+def test_gemv_cluster_cut_steps_with_stale_memory(q):
+    # what other launches left in shared memory (all bits set: NaN as scales)
+    # has no part in a cut step
+    w = inputs.student_t_weights_cuda(64, 1024, 11, outliers=False)
+    full = sss.sss_quantize(w, q, 32, sss.GRID_ASYM)
+    full.codes.fill_(255)
+    full.scales.fill_(-1)
+    full.mins.fill_(-1)
+    cut = sss.sss_quantize(w[:, :864].contiguous(), q, 32, sss.GRID_ASYM)
+    x = inputs.normal_bf16_cuda((16, 1024), 12)
+    xc = x[:, :864].contiguous()
+    ref = xc.double() @ sss.sss_dequantize(cut).double().T
+    for _ in range(20):
+        sss.sss_gemv(full, x)
+        y = sss.sss_gemv(cut, xc)
+        assert ((y - ref).abs().amax(1) / ref.abs().amax(1)).max().item() <= TOL
