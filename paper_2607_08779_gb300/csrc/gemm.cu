@@ -39,9 +39,10 @@
 // column).
 // What bounds it: at BN = 256 the MMAs (1025 cycles a step; 512 per k-block is
 // the pipe's rate), 86 % of cuBLAS's burst rate at 2048 tokens with the
-// conversion of X (14336 x 4096 q = 4: 145 us; 192 us when a tile's k-blocks
-// each brought their own narrow code and scale tiles); at BN <= 128 the
-// dequantisation (590-730 cycles a step); at few tokens the launch itself.
+// conversion of X (14336 x 4096 q = 4: 144 us; 192 us when a tile's k-blocks
+// each brought their own narrow code and scale tiles); at BN <= 128 the TMA
+// unit's rows and the way from L2 to the SM (650-750 cycles a step; the MMAs
+// need 512 at BN = 128); at few tokens the launch itself.
 // Every mbarrier wait is bounded (about one second of global time); on
 // expiry the CTA raises SSS_FLAG_TIMEOUT, all roles leave their loops, and
 // the tensor memory is still released.
@@ -1086,8 +1087,8 @@ size_t split_bytes(int64_t rt, int64_t m, const GemmPlan& p) {
 
 // The plan of least estimated time, in SM cycles: each SM's share of the items,
 // an item at a time, plus the launch's start and end, and for K splits the last
-// arrival's sum of the partial tiles.  Per k-block 64- and 128-token tiles take
-// about 290 cycles (the dequantisation's rate) and 256-token tiles 512 (the
+// arrival's sum of the partial tiles.  Per k-block 64- and 128-token tiles count
+// about 290 cycles (325-375 in a long loop) and 256-token tiles 512 (the
 // MMAs').  Splits end on code-tile boundaries and keep at least 8 k-blocks.
 // rt: the row tiles of all the call's matrices; ws: the bytes the partial tiles
 // must fit in.  K is split only to fill SMs that the tiles leave idle.

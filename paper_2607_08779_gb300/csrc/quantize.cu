@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(kRotThreads)
 // of 8192) is a pass of its own.  So the chunk crosses shared memory five
 // times for any block up to 4096, where a butterfly at a time crossed it
 // twelve times with an integer division each (14336 x 4096, q = 3, blocks of
-// 4096: 419 us; this takes 96 us, 2.7 TB/s).
+// 4096: 419 us; this takes 93 us, 2.8 TB/s).
 // The pass over consecutive values reads the 16-byte pieces c of its 256 bytes
 // in the order c ^ (t & 7), which keeps a quarter-warp's banks distinct; a
 // butterfly between pieces then finds its lower element in either of two
