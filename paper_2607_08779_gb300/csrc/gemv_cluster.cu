@@ -171,6 +171,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int share = NBC * kRows / S;        // outputs of a tile per CTA
   const int my_tiles = cid < a.ntiles ? (a.ntiles - cid + nclus - 1) / nclus : 0;
 
+  // "this CTA has started": the peers store into its shared memory, which they
+  // may do only once they know that it runs
+  if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -351,6 +354,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       xput(ul, nr);
     }
   __syncthreads();
+  // every CTA of the cluster has started (long since: the staging lies between)
+  if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
   float acc[2][NBLK][4];
 #pragma unroll

@@ -1,0 +1,32 @@
+"""Order of the synchronising instructions inside the kernels, read from their
+source: what a run cannot show, because it comes out right by timing."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2607_08779_gb300", "csrc")
+
+
+def kernel_text(file, name):
+    """The body of the function `name` in csrc/`file`, without comments."""
+    with open(os.path.join(CSRC, file)) as f:
+        src = f.read()
+    src = re.sub(r"/\*.*?\*/", "", re.sub(r"//[^\n]*", "", src), flags=re.S)
+    start = src.index("{", src.index(" " + name + "("))
+    depth = 0
+    for i in range(start, len(src)):
+        depth += {"{": 1, "}": -1}.get(src[i], 0)
+        if depth == 0:
+            return src[start:i + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def test_cluster_gemv_waits_for_its_peers_before_remote_stores():
+    # another CTA's shared memory exists only once that CTA has started: every
+    # thread arrives at the cluster barrier on entry and waits for it before
+    # the first store into a peer
+    body = kernel_text("gemv_cluster.cu", "gemv_cluster_kernel")
+    arrive = body.index("barrier.cluster.arrive.relaxed.aligned")
+    wait = body.index("barrier.cluster.wait.acquire.aligned")
+    assert arrive < wait < body.index("st.shared::cluster")
+    assert wait < body.index("cluster.sync()")
