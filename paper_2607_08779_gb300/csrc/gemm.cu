@@ -396,7 +396,14 @@ constexpr int kAStages = 4; // A operand steps (two k-blocks) in tensor memory
 // whoever waits on one has to wait for every phase in turn.  The dequantising
 // groups take every fourth step and every other code tile: the A stages are a
 // multiple of four and the code tiles an even number, which gives each group
-// stages of its own.
+// stages of its own.  The A stages go by step number, of which an item of an odd
+// number of steps leaves one out.  Four activation stages (JOINT) go by it too, so
+// that a step has one stage for both operands.  Three go step after step and are
+// freed by the A stages' barriers: the producer looks at every step's in turn, and
+// runs no further ahead than an A stage comes round again (two steps where every
+// other number is left out).  (Barriers of their own took a second commit per
+// step, 2.8 % of a 256-token tile; the look-ahead rule for four stages as well 15 %
+// of down_proj at 512 tokens, where the producer sets the pace.)
 
 // Shared memory: XS activation tiles (1024-aligned for the 128-byte
 // swizzle), then with CT the code tiles, then the barriers.
@@ -408,11 +415,12 @@ struct Smem {
   static constexpr int W_BYTES = CT ? kBM * 32 * Q : 0;
   static constexpr int W_OFF = XS * 2 * X_BYTES;
   static constexpr int BAR_OFF = W_OFF + WS * W_BYTES;
+  static constexpr bool JOINT = XS == kAStages;              // one stage for X and A
   static constexpr int NB = BN == 256 ? 1 : 2;               // accumulators
   static constexpr int NBAR = XS + 2 * kAStages + 2 * WS + 2 * NB + 1;
   static constexpr int TOTAL = BAR_OFF + NBAR * 8 + 16 + 1024;  // + align slack
   static constexpr int A_COL = NB * BN;           // first A-stage column in tensor memory
-  static_assert(kAStages % 4 == 0 && WS % 2 == 0 && XS <= kAStages, "see kAStages");
+  static_assert(kAStages == 4 && WS % 2 == 0 && XS <= kAStages, "see kAStages");
   static_assert(TOTAL <= 227 * 1024, "shared memory per CTA");
   static_assert(NB * BN + 64 * kAStages <= 512, "tensor memory holds accumulators and A stages");
 };
@@ -635,9 +643,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ---------------- TMA producer: activation and code tiles ----------------
     int sx = 0, xn = 0;      // activation stage, and how many steps were issued
     int sw = 0, wn = 0;      // code stage, and how many tiles were issued
-    uint32_t phx = 0, phw = 0;
+    uint32_t phw = 0;
+    uint32_t usedx = 0;      // bit s: the parity of activation stage s's next use
+    // unless JOINT
     uint32_t used = 0;       // bit s: the parity of A stage s's next use
     uint32_t hist = 0;       // the last steps' A stages and parities, 4 bits each
+    uint32_t near = 0;       // bit i: step number P + p - 1 - i is a step, i = 0 .. 3
+    int seen = 0;            // steps whose MMAs are known to have completed
     int P = 0;
     bool ok = true;
     for (int it = blockIdx.x; it < a.items && ok; it += gridDim.x) {
@@ -669,15 +681,22 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        // the stage is free once the MMAs of XS steps ago have completed
-        if (xn >= XS) {
-          const uint32_t h = hist >> (4 * (XS - 1));
-          const bool freed = mbar_wait(&empty[(h >> 1) & 3u], h & 1u, abort);
-          if (!__all_sync(0xffffffffu, freed)) {
-            ok = false;
-            break;
+        if constexpr (S::JOINT) {
+          // the stage is free once the MMAs that used it last have completed
+          const bool freed = mbar_wait(&empty[sx], ((usedx >> sx) & 1u) ^ 1u, abort);
+          ok = __all_sync(0xffffffffu, freed);
+        } else {
+          // the stage is free once the MMAs of XS steps ago have completed; and
+          // the last step of this A stage has to be seen before this one can
+          // complete the barrier's next phase
+          const int ahead = (near & 8u) ? min(XS, __popc(near)) : XS;
+          for (; xn - seen >= ahead && ok; ++seen) {
+            const uint32_t h = hist >> (4 * (xn - seen - 1));
+            const bool freed = mbar_wait(&empty[(h >> 1) & 3u], h & 1u, abort);
+            ok = __all_sync(0xffffffffu, freed);
           }
         }
+        if (!ok) break;
         if (elect_one()) {
           // (a box past the end of k reads zeros)
           unsigned char* dst = smem + sx * 2 * S::X_BYTES;
@@ -688,22 +707,28 @@ __global__ void __launch_bounds__(kThreads, 1)
                       w.m0);
         }
         __syncwarp();
-        const uint32_t sa = static_cast<uint32_t>(P + p) & 3u;
-        hist = (hist << 4) | (sa << 1) | ((used >> sa) & 1u);
-        used ^= 1u << sa;
-        if (++sx == XS) {
-          sx = 0;
-          phx ^= 1u;
-        }
+        usedx ^= 1u << sx;
+        if (++sx == XS) sx = 0;
         ++xn;
+        if constexpr (!S::JOINT) {
+          const uint32_t sa = static_cast<uint32_t>(P + p) & 3u;
+          hist = (hist << 4) | (sa << 1) | ((used >> sa) & 1u);
+          used ^= 1u << sa;
+          near = ((near << 1) | 1u) & 15u;
+        }
+      }
+      if (w.nsteps & 1) {  // the step number left out
+        if (S::JOINT) sx = (sx + 1) & 3;
+        near = (near << 1) & 15u;
       }
       P += (w.nsteps + 1) & ~1;
     }
     if (*abort) {
-      // let this CTA's copies still in flight land before the CTA exits
+      // let this CTA's copies still in flight land before the CTA exits (of a
+      // stage never used, the phase before its first counts as completed)
       int drain = 0;
-      for (int i = max(0, xn - XS); i < xn; ++i)
-        (void)mbar_wait(&full_x[i % XS], static_cast<uint32_t>(i / XS) & 1u, &drain);
+      for (int s = 0; s < XS; ++s)
+        (void)mbar_wait(&full_x[s], ((usedx >> s) & 1u) ^ 1u, &drain);
       for (int i = max(0, wn - WS); i < wn; ++i)
         (void)mbar_wait(&full_w[i % WS], static_cast<uint32_t>(i / WS) & 1u, &drain);
     }
@@ -736,7 +761,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (P0 + s < P || P0 + s >= end || !go) continue;
           if (!there) {
             bool t = mbar_wait(&full_a[s], (used >> s) & 1u, abort);
-            t = t && mbar_wait(&full_x[sx], phx, abort);
+            t = t && mbar_wait(&full_x[S::JOINT ? s : sx], S::JOINT ? (used >> s) & 1u : phx, abort);
             if (!__all_sync(0xffffffffu, t)) {
               go = false;
               continue;
@@ -744,14 +769,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           used ^= 1u << s;
           tc_fence_after();
-          const uint64_t bd = bdesc0 + 2 * bstep * sx;
-          if (++sx == XS) {
+          const uint64_t bd = bdesc0 + 2 * bstep * (S::JOINT ? s : sx);
+          if (!S::JOINT && ++sx == XS) {
             sx = 0;
             phx ^= 1u;
           }
           constexpr int kNext[4] = {1, 2, 3, 0};
           const bool next = mbar_test_wait(&full_a[kNext[s]], (used >> kNext[s]) & 1u) &&
-                            mbar_test_wait(&full_x[sx], phx);
+                            mbar_test_wait(&full_x[S::JOINT ? kNext[s] : sx],
+                                           S::JOINT ? (used >> kNext[s]) & 1u : phx);
           if (elect_one()) {
             const uint32_t ta = tm + static_cast<uint32_t>(S::A_COL + 64 * s);
             umma_kblock(acc, ta, bd, idesc, P0 + s == P ? 1u : 0u);

@@ -20,6 +20,8 @@ from test_gpu_gemm import run_case  # noqa: E402
     (3, 32, 384, sss.GRID_UNSIGNED_SYM),  # 3 steps, 96-byte code tiles
     (2, 128, 384, sss.GRID_ASYM),         # 3 steps, one scale each
     (2, 64, 64, sss.GRID_SIGNED_SYM),     # a single k-block
+    (4, 64, 128, sss.GRID_SIGNED_SYM),    # a single step
+    (2, 32, 1152, sss.GRID_UNSIGNED_SYM),  # 9 steps
 ])
 def test_gemm_several_tiles_per_cta(q, g, k, grid, m):
     # 157 row tiles: more than the SMs, the last one ragged
