@@ -180,7 +180,10 @@ sss_status_t sss_gemv(const sss_qtensor_t* qt, const uint16_t* x_bf16,
                                        kernel has completed                                */
 #define SSS_GEMV_WEIGHTS_READY 0x2u /* with SSS_GEMV_PDL: the packed weights are not written
                                        by the preceding work in the stream, so they may be
-                                       streamed in before it completes                     */
+                                       streamed in before it completes.  (What may still be
+                                       running: the call before this one, and while that is
+                                       a sss_gemv_multi with this flag, the call before it
+                                       as well.)                                           */
 #define SSS_GEMV_ACT_Q8 0x4u        /* quantize x to Q8_0 on the fly (see
                                        sss_quantize_act_q8) and multiply the packed
                                        weights with the Q8_0 values: y_j[r] =

@@ -161,7 +161,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_batch_kernel(const __grid_co
                      : "memory");
     }
   }
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const int64_t tstride = static_cast<int64_t>(gridDim.x) * ngrp;
   const int64_t tfirst = static_cast<int64_t>(grp) * gridDim.x + blockIdx.x;
@@ -354,8 +353,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_batch_kernel(const __grid_co
   // well under a microsecond, but the shared-memory stores of its
   // conversion would otherwise wait behind the ring's DRAM loads in the
   // SM's load/store queue.  The barrier comes before the ring's loads too,
-  // so no warp waits for another warp's loads to be issued.
+  // so no warp waits for another warp's loads to be issued.  The next kernel
+  // may start only now: one that reads its weights early then finds written
+  // what the launches before this one wrote.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   stage_from(std::integral_constant<int, 4>{}, 0, threadIdx.x);
   __syncthreads();
   Regs ring[D];

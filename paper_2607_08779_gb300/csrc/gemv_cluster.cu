@@ -174,8 +174,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   // "this CTA has started": the peers store into its shared memory, which they
   // may do only once they know that it runs
   if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // in this order: a next kernel that reads its weights early then finds written
+  // what the launches before this one wrote
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // ---- the warp's stream: its steps of tiles grp, grp + ngrp, ... of the
   // cluster's (tile j of the cluster is tile cid + j nclus) ----

@@ -277,8 +277,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
 
   if (threadIdx.x >= 32 && threadIdx.x < 64)
     reinterpret_cast<uint32_t*>(xs + zoff)[threadIdx.x - 32] = 0u;  // the zero blocks
-  // allow the next kernel in the stream to be scheduled as SMs free up
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // allow the next kernel in the stream to be scheduled as SMs free up: with
+  // early weights at once, else only when everything before this kernel has
+  // completed, so that a next one that reads its weights early finds written
+  // what the launches before this one wrote
+  if (a.early_weights) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // ---- this warp's stream: tiles t = (i * ngrp + grp) * gridDim.x + blockIdx.x,
   // i = 0, 1, ... (consecutive tiles go to different SMs, so every SM gets
@@ -393,7 +396,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_stream_kernel(const __grid_c
 
   Regs ring[D];
   set_tile(0);
-  if (!a.early_weights) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!a.early_weights) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
 #pragma unroll
   for (int d = 0; d < D; ++d)
     if (d < total) fetch(ring[d]);

@@ -372,10 +372,11 @@ __global__ void __launch_bounds__(kQThreads, 1)
   }
   // Launched as a programmatic dependent launch: the set-up above may run
   // while the preceding kernel drains; no global memory is touched before
-  // that kernel has completed.  The next kernel may be scheduled at once
-  // (it, in turn, waits for this one before it reads what this writes).
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // that kernel has completed.  Only then may the next kernel be scheduled
+  // (it, in turn, waits for this one before it reads what this writes): one
+  // that reads its weights early finds written what was launched before this.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();
 
   if (warp == 0) {
@@ -681,8 +682,8 @@ __device__ __forceinline__ void rotate_rows_ring(const float* __restrict__ w, in
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // a programmatic dependent launch, as quantize_kernel
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
     if (lane == 0) {

@@ -147,3 +147,30 @@ def test_stream_activation_scale_varies_per_chunk(q, g):
     the dot product, the small ones must not be lost or overflow."""
     check_scaled_x(300, 4096, q, g, sss.GRID_SIGNED_SYM, 90 + q + g,
                    lambda i: 10.0 ** ((i * 7) % 13 - 8))
+
+
+def _middle_call(kind, qts, x, w):
+    if kind == "quantize_rotated":
+        sss.sss_quantize_rotated(w, 64, 4, 32, sss.GRID_SIGNED_SYM, out=qts[4])
+    else:
+        q, batch = {"gemv": (4, 1), "gemv q=4 batch 4": (4, 4), "gemv q=3 batch 4": (3, 4)}[kind]
+        sss.sss_gemv(qts[q], x[:batch])
+
+
+@pytest.mark.parametrize("kind", ["gemv", "gemv q=4 batch 4", "gemv q=3 batch 4", "quantize_rotated"])
+def test_weights_written_two_calls_before(kind):
+    # WEIGHTS_READY speaks of the call before: what the one before that writes
+    # (here the quantizer) is complete when the weights are read
+    n, k = 8192, 4096
+    small = inputs.student_t_weights_cuda(16, 512, 1, outliers=False)
+    qts = {q: sss.sss_quantize(small, q, 32, sss.GRID_SIGNED_SYM) for q in (3, 4)}
+    xs = inputs.normal_bf16_cuda((4, 512), 2)
+    x = inputs.normal_bf16_cuda((k,), 3)
+    ws = [inputs.student_t_weights_cuda(n, k, s, outliers=False) for s in (4, 5)]
+    want = [sss.sss_gemv_multi([sss.sss_quantize(w, 4, 32, sss.GRID_SIGNED_SYM)], x)[0] for w in ws]
+    out = sss.empty_qtensor(n, k, 4, 32, sss.GRID_SIGNED_SYM)
+    for i in range(20):
+        sss.sss_quantize(ws[i % 2], 4, 32, sss.GRID_SIGNED_SYM, out=out)
+        _middle_call(kind, qts, xs, small)
+        y = sss.sss_gemv_multi([out], x, flags=sss.GEMV_PDL | sss.GEMV_WEIGHTS_READY)[0]
+        assert torch.equal(y, want[i % 2])

@@ -3,6 +3,8 @@ source: what a run cannot show, because it comes out right by timing."""
 import os
 import re
 
+import pytest
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_2607_08779_gb300", "csrc")
 
@@ -30,3 +32,25 @@ def test_cluster_gemv_waits_for_its_peers_before_remote_stores():
     wait = body.index("barrier.cluster.wait.acquire.aligned")
     assert arrive < wait < body.index("st.shared::cluster")
     assert wait < body.index("cluster.sync()")
+
+
+@pytest.mark.parametrize("file,name", [
+    ("gemv_cluster.cu", "gemv_cluster_kernel"),
+    ("gemv_batch.cu", "gemv_batch_kernel"),
+    ("quantize.cu", "quantize_kernel"),
+    ("quantize.cu", "rotate_rows_ring"),
+])
+def test_the_next_kernel_starts_only_behind_the_wait(file, name):
+    # a sss_gemv_multi with SSS_GEMV_WEIGHTS_READY reads its weights as soon as it
+    # starts: were it let in before this kernel's wait, they might still be being
+    # written by the launch before this one
+    body = kernel_text(file, name)
+    assert body.index("griddepcontrol.wait") < body.index("griddepcontrol.launch_dependents")
+
+
+def test_the_streaming_gemv_lets_the_next_kernel_in_early_only_with_early_weights():
+    body = re.sub(r"\s+", " ", kernel_text("gemv_stream.cu", "gemv_stream_kernel"))
+    release = 'asm volatile("griddepcontrol.launch_dependents;" ::: "memory");'
+    assert body.count(release) == 2
+    assert "if (a.early_weights) " + release in body
+    assert 'if (!a.early_weights) { asm volatile("griddepcontrol.wait;" ::: "memory"); ' + release in body
