@@ -148,8 +148,10 @@ sss_status_t sss_dequantize(const sss_qtensor_t* qt, void* out,
  * symmetric formats, plus the row-sum term sum_b m * sum_{k in b} x for
  * ASYM).  fp32 accumulation; deterministic (no atomics).  At batch 1, and at
  * batch 2..16 for q = 2 and 4, the integer codes meet the activations exactly
- * (activations within fp16's range) and the group scale is applied in fp32;
- * so too for q = 3 with k not a multiple of 256.  Otherwise, for q = 3, the
+ * and the group scale is applied in fp32; so too for q = 3 with k not a multiple
+ * of 256.  (At batch 2..16 an activation enters as fp16 x * 2^-p, p = 0, 2 or 4
+ * the bit offset of the code's field: exactly x for 2^-13 <= |x| <= 65504, below
+ * that within 2^-21 of it.)  Otherwise, for q = 3, the
  * batch fills the tensor-core columns across groups, so each weight enters the
  * product as w^ rounded once to fp16 (<= 2^-11 relative, as in sss_gemm), times
  * 2^p (p = 0, 2 or 4, the bit offset of the code's field).  That operand fits

@@ -318,10 +318,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         f[2 * e] = __uint_as_float(wv[e] << 16);
         f[2 * e + 1] = __uint_as_float(wv[e] & 0xFFFF0000u);
       }
-      float sum = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
-#pragma unroll
-      for (int o = 1; o < G / 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if (st >= ns || r >= a.batch) continue;
       uint32_t pr[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -331,7 +327,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float mul = kMul[Q == 4 ? 0 : 1][e];
         __half2 hv = __floats2half2_rn(f[e] * mul, f[e + 4] * mul);
         pr[e] = *reinterpret_cast<uint32_t*>(&hv);
+        // x as the operand holds it (exactly x from 2^-13 on): the row sum has to
+        // meet the codes' product with the same values, or what fp16 rounded off
+        // smaller ones would be left over times 2^(q-1)
+        const float2 held = __half22float2(hv);
+        f[e] = held.x * (1.f / mul);
+        f[e + 4] = held.y * (1.f / mul);
       }
+      float sum = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
+#pragma unroll
+      for (int o = 1; o < G / 8; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (st >= ns || r >= a.batch) continue;
       const uint32_t dst = dst0 + static_cast<uint32_t>((r >> 3) * 512 + (r & 7) * 64);
       asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(pr[0]), "r"(pr[1]),
                    "r"(pr[2]), "r"(pr[3])

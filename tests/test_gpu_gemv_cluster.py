@@ -86,3 +86,22 @@ def test_gemv_cluster_cut_steps_with_stale_memory(q):
         sss.sss_gemv(full, x)
         y = sss.sss_gemv(cut, xc)
         assert ((y - ref).abs().amax(1) / ref.abs().amax(1)).max().item() <= TOL
+
+
+@pytest.mark.parametrize("k", [512, 544])  # whole steps, and a last one cut short
+@pytest.mark.parametrize("q,grid", [(4, sss.GRID_SIGNED_SYM), (2, sss.GRID_UNSIGNED_SYM), (4, sss.GRID_ASYM)])
+@pytest.mark.parametrize("mag", [1e-8, 1e-6, 1e-5, 1e-4])
+def test_gemv_cluster_small_activations(mag, q, grid, k):
+    # below 2^-13 the operand fl16(x 2^-p) holds x rounded; the product has to be
+    # that of the rounded values, symmetric offset and minimum included
+    qt = sss.sss_quantize(inputs.student_t_weights_cuda(100, k, 13, outliers=False), q, 32, grid)
+    x = (inputs.normal_bf16_cuda((5, k), 14).float() * mag).bfloat16()
+    pos = torch.tensor([0., 4., 0., 4.] if q == 4 else [0., 2., 4., 0.], device="cuda")
+    p2 = torch.exp2(pos.repeat(k // 4))  # of elements e and e + 4 of every eight
+    held = (x.float() / p2).half().double() * p2.double()
+    w = sss.sss_dequantize(qt).double()
+    # an output is a chain of at most 40 fp32 or tensor-core additions, each off by
+    # 2^-23 of the magnitudes that it adds: codes are up to 2^q <= 16 steps, so a
+    # term is up to 16 max|w| |x|
+    bound = 40 * 2.0**-23 * (held.abs().sum(1, keepdim=True) * 16 * w.abs().amax(1))
+    assert ((sss.sss_gemv(qt, x) - held @ w.T).abs() <= bound).all()
