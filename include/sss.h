@@ -151,7 +151,9 @@ sss_status_t sss_dequantize(const sss_qtensor_t* qt, void* out,
  * and the group scale is applied in fp32; so too for q = 3 with k not a multiple
  * of 256.  (At batch 2..16 an activation enters as fp16 x * 2^-p, p = 0, 2 or 4
  * the bit offset of the code's field: exactly x for 2^-13 <= |x| <= 65504, below
- * that within 2^-21 of it.)  Otherwise, for q = 3, the
+ * that within 2^-21 of it.  For q = 2 and 4 the outputs of a batch row with larger
+ * or infinite activations are computed by plain fp32 products of w^ and x, many
+ * times slower; for q = 3 they are infinite or NaN.)  Otherwise, for q = 3, the
  * batch fills the tensor-core columns across groups, so each weight enters the
  * product as w^ rounded once to fp16 (<= 2^-11 relative, as in sss_gemm), times
  * 2^p (p = 0, 2 or 4, the bit offset of the code's field).  That operand fits

@@ -105,3 +105,26 @@ def test_gemv_cluster_small_activations(mag, q, grid, k):
     # term is up to 16 max|w| |x|
     bound = 40 * 2.0**-23 * (held.abs().sum(1, keepdim=True) * 16 * w.abs().amax(1))
     assert ((sss.sss_gemv(qt, x) - held @ w.T).abs() <= bound).all()
+
+
+@pytest.mark.parametrize("n,k", [(100, 1024), (300, 4352), (70, 544)])
+@pytest.mark.parametrize("q,grid", [(4, sss.GRID_SIGNED_SYM), (2, sss.GRID_SIGNED_SYM),
+                                    (2, sss.GRID_ASYM), (4, sss.GRID_ASYM)])
+def test_gemv_cluster_activations_beyond_fp16(q, grid, n, k):
+    qt = sss.sss_quantize(inputs.student_t_weights_cuda(n, k, 15, outliers=False), q, 32, grid)
+    x = inputs.normal_bf16_cuda((16, k), 16)
+    plain = sss.sss_gemv(qt, x)
+    x[1] *= 65536.0           # many from 65520 on
+    x[2, 5] = 1e30            # one, of any size
+    x[7, k - 1] = float("inf")
+    x[9, 0] = float("-inf")
+    x[15, 3] = float("nan")
+    y = sss.sss_gemv(qt, x)
+    ref = x.double() @ sss.sss_dequantize(qt).double().T
+    same = [b for b in range(16) if b not in (1, 2, 7, 9, 15)]
+    assert torch.equal(y[same], plain[same])
+    for b in (1, 2):
+        assert ((y[b] - ref[b]).abs().max() / ref[b].abs().max()).item() <= TOL
+    for b in (7, 9, 15):  # +-inf by the weight's sign, NaN where it is zero
+        assert torch.equal(y[b].isnan(), ref[b].isnan())
+        assert torch.equal(y[b].nan_to_num(0.0), ref[b].float().nan_to_num(0.0))
