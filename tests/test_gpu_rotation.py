@@ -78,6 +78,16 @@ def test_quantize_rotated_ragged_last_chunk():
     assert np.array_equal(qt.scales.cpu().numpy().view(np.uint16), scales)
 
 
+@pytest.mark.parametrize("n,k,b", [(1, 4, 2), (7, 1536, 512), (301, 8192 + 4096, 4096)])
+def test_rotate_rows_ragged_last_chunk(n, k, b):
+    # the last chunk of 8192 values partial (one value group at least, in place);
+    # 452 chunks: two rounds of some groups of warps
+    W = inputs.student_t_weights(n, k, 440 + b, outliers=False)
+    w = to_dev(W)
+    sss.sss_hadamard(w, b, sss.ROTATE_INPUT, out=w)
+    assert np.array_equal(w.cpu().numpy().view(np.uint32), oracle.rotate(W, b, "rows").view(np.uint32))
+
+
 def test_rotation_rejects_bad_blocks():
     w = torch.zeros((8, 96), dtype=torch.float32, device="cuda")
     for b in (0, 3, 64, 16384):  # not a power of two, not dividing k, too large

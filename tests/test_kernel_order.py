@@ -39,6 +39,7 @@ def test_cluster_gemv_waits_for_its_peers_before_remote_stores():
     ("gemv_batch.cu", "gemv_batch_kernel"),
     ("quantize.cu", "quantize_kernel"),
     ("quantize.cu", "rotate_rows_ring"),
+    ("quantize.cu", "hadamard_rows_kernel"),
 ])
 def test_the_next_kernel_starts_only_behind_the_wait(file, name):
     # a sss_gemv_multi with SSS_GEMV_WEIGHTS_READY reads its weights as soon as it
@@ -54,3 +55,11 @@ def test_the_streaming_gemv_lets_the_next_kernel_in_early_only_with_early_weight
     assert body.count(release) == 2
     assert "if (a.early_weights) " + release in body
     assert 'if (!a.early_weights) { asm volatile("griddepcontrol.wait;" ::: "memory"); ' + release in body
+
+
+@pytest.mark.parametrize("name", ["hadamard_rows_kernel", "hadamard_cols_kernel"])
+def test_the_rotation_without_a_status_has_no_wait_that_can_expire(name):
+    # sss_hadamard takes no status word: an expired wait would go unreported
+    body = kernel_text("quantize.cu", name)
+    for called in ("q_wait", "rotate_rows_ring", "mbarrier"):
+        assert called not in body
