@@ -17,9 +17,9 @@
 //           zero halves s instead);
 //   then the codes of the refined scale by the quantizer's exact-quotient
 //   rounding, packed in the library's layout, with the fp16 scale.
-// G/32 lanes own a group, 32 elements each (lane l elements l + e G/32), so
-// the pairwise sum is a tree in registers and its last log2(G/32) levels are
-// shuffles -- the order above, bit for bit.
+// In lsq_kernel G/32 lanes own a group, 32 elements each (lane l elements
+// l + e G/32), so the pairwise sum is a tree in registers and its last log2(G/32)
+// levels are shuffles -- the order above, bit for bit.
 //
 // Bound by instruction issue (65 % of the slots, the rest waiting on the ALU and
 // FMA pipes): a step takes about 12 instructions per weight.
@@ -31,7 +31,7 @@
 // to RN(w / s)), which holds while nothing underflows; a group or step
 // outside that range divides.  (One warp per group, a division per weight
 // and five dependent shuffles per step took 567 us for 20 steps on 4096 x
-// 4096 at q = 4, g = 32; this takes 170 us.)
+// 4096 at q = 4, g = 32; this takes 170 us.  Few groups still go that way.)
 #include <math.h>
 
 #include <algorithm>
@@ -301,30 +301,174 @@ __global__ void __launch_bounds__(kLsqThreads)
   }
 }
 
+// The same with a warp per group, for few groups: lane l holds elements l + 32 e,
+// so the in-lane levels of the pairwise sum come first and the last five are
+// shuffles.  More instructions per weight (a division, and the shuffles for one to
+// four weights), but a step takes 0.2 us where 32 weights in a row take 0.7.
+template <int Q, bool SIGNED, int G>
+__global__ void __launch_bounds__(kLsqThreads)
+    lsq_warp_kernel(const float* __restrict__ w, int64_t ngroups, int steps, float step,
+                    uint8_t* __restrict__ codes, uint16_t* __restrict__ scales,
+                    uint32_t* __restrict__ status) {
+  constexpr int E = G / 32;  // elements per lane
+  constexpr int HALF = 1 << (Q - 1);
+  constexpr float QN = -static_cast<float>(HALF), QP = static_cast<float>(HALF - 1);
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = static_cast<int64_t>(gridDim.x) * (kLsqThreads / 32);
+  for (int64_t grp = static_cast<int64_t>(blockIdx.x) * (kLsqThreads / 32) + (threadIdx.x >> 5);
+       grp < ngroups; grp += warps) {  // warp-uniform
+    float x[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] = __ldcs(w + grp * G + lane + 32 * e);
+    // the (signed) absmax scale, as the quantizer forms it
+    float mx = x[0], mn = x[0];
+    unsigned bad = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      mx = fmaxf(mx, x[e]);
+      mn = fminf(mn, x[e]);
+      bad |= is_nonfinite(x[e]);
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      bad |= __shfl_xor_sync(0xffffffffu, bad, o);
+    }
+    const float M = fmaxf(mx, -mn);
+    const float gamma = (SIGNED && mx > -mn) ? -1.f : 1.f;
+    const float alpha = __fmul_rn(M, 1.0f / HALF);
+    const bool zero = (alpha == 0.f) || bad;
+    float s = zero ? 0.f : gamma * alpha;
+    // ---- LSQ steps ----
+    if (!zero) {
+      for (int it = 0; it < steps; ++it) {
+        float t[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const float v = __fdiv_rn(x[e], s);
+          float c, d;
+          if (v <= QN) {
+            c = QN;
+            d = QN;
+          } else if (v >= QP) {
+            c = QP;
+            d = QP;
+          } else {
+            c = fminf(fmaxf(rintf(v), QN), QP);
+            d = __fsub_rn(c, v);
+          }
+          const float err = __fsub_rn(__fmul_rn(s, c), x[e]);
+          t[e] = __fmul_rn(__fmul_rn(2.f, err), d);
+        }
+#pragma unroll
+        for (int h = E / 2; h >= 1; h >>= 1)
+#pragma unroll
+          for (int e = 0; e < h; ++e) t[e] = __fadd_rn(t[e], t[e + h]);
+        float gsum = t[0];
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) gsum = __fadd_rn(gsum, __shfl_xor_sync(0xffffffffu, gsum, o));
+        float sn = __fsub_rn(s, __fmul_rn(step, gsum));
+        if (__fmul_rn(sn, s) <= 0.f) sn = __fmul_rn(s, 0.5f);
+        s = sn;
+      }
+    }
+    // ---- codes of the refined scale (exact-quotient rounding) ----
+    int u[E];
+    if (zero) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) u[e] = HALF;
+    } else {
+      float ss = s, sig = 1.f;
+      const float as = fabsf(s) * static_cast<float>(HALF);  // about ||w||_inf
+      if (as < 0x1p-96f || as > 0x1p+96f) {  // keep 1/s normal: scale w and s by 2^+-64
+        sig = (as < 1.f) ? 0x1p+64f : 0x1p-64f;
+        ss = __fmul_rn(s, sig);
+      }
+      const float r = __frcp_rn(ss);
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int up = code_of<HALF>(sig == 1.f ? x[e] : __fmul_rn(x[e], sig), ss, r);
+        u[e] = max(0, min(up, 2 * HALF - 1));
+      }
+    }
+    const uint16_t s16 = __half_as_ushort(__float2half_rn(s));
+    // ---- pack: element l + 32 e is code l of run e of the group ----
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      if constexpr (Q == 4) {  // run e: 4 words, word l/8 holds codes 8(l/8) .. +7
+        uint32_t v = static_cast<uint32_t>(u[e]) << (4 * (lane & 7));
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 7) == 0)
+          reinterpret_cast<uint32_t*>(codes + grp * (G / 2) + 16 * e)[lane >> 3] = v;
+      } else if constexpr (Q == 2) {  // run e: 2 words, word l/16 holds codes 16(l/16) .. +15
+        uint32_t v = static_cast<uint32_t>(u[e]) << (2 * (lane & 15));
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
+        if ((lane & 15) == 0)
+          reinterpret_cast<uint32_t*>(codes + grp * (G / 4) + 8 * e)[lane >> 4] = v;
+      } else {  // q = 3: run e's low-plane words 2e, 2e+1; high-plane word G/16 + e
+        uint32_t v = static_cast<uint32_t>(u[e] & 3) << (2 * (lane & 15));
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
+        const uint32_t hi = __ballot_sync(0xffffffffu, (u[e] >> 2) & 1);
+        uint32_t* base = reinterpret_cast<uint32_t*>(codes + grp * (3 * G / 8));
+        if ((lane & 15) == 0) base[2 * e + (lane >> 4)] = v;
+        if (lane == 0) base[G / 16 + e] = hi;
+      }
+    }
+    if (lane == 0) {
+      scales[grp] = s16;
+      unsigned flags = bad ? SSS_FLAG_NONFINITE : 0u;
+      if ((s16 & 0x7fffu) == 0x7c00u) flags |= SSS_FLAG_RANGE;
+      if (flags != 0u && status != nullptr) atomicOr(status, flags);
+    }
+  }
+}
+
+// Whether a warp per group takes less time than 32 weights per thread: both in us
+// as measured over 64 .. 16384 x 1024 with 0 .. 50 steps.  Where the lines cross
+// (in 2^20 weights): groups of 32, 0.9 without steps and 0.45 at 20; of 128, 5 and
+// 0.65.  (20 steps at q = 4, g = 32: 64 x 1024 6.4 us against 19.3, 256 x 1024 12.1
+// against 19.6, 512 x 1024 21.5 against 19.4, 4096 x 1024 141 against 54.)
+bool few_groups(int64_t weights, int group, int steps) {
+  const double m = static_cast<double>(weights) / (1 << 20);
+  const int64_t sms = device_sm_count(), blocks = (weights / 32 + kLsqThreads - 1) / kLsqThreads;
+  const double waves = static_cast<double>((blocks + sms - 1) / sms);
+  const double base = group == 32 ? 4.6 : (group == 64 ? 3.0 : 2.0);
+  const double per_step = group == 32 ? 1.55 : (group == 64 ? 1.35 : 1.15);
+  const double start = group == 64 ? 5.0 + 2.1 * waves : 4.5 + 1.6 * waves;
+  return 2.3 + m * (base + per_step * steps) < start + (0.18 + 0.49 * waves) * steps;
+}
+
+template <int Q, bool SIGNED, int G>
+cudaError_t lsq_run(const float* w, const sss_qtensor_t& t, int steps, float step,
+                    uint32_t* status, cudaStream_t stream) {
+  const int64_t ngroups = t.n * (t.k / G);
+  const bool few = few_groups(ngroups * G, G, steps);
+  const int64_t threads = ngroups * (few ? 32 : G / 32);
+  const int64_t want = (threads + kLsqThreads - 1) / kLsqThreads;
+  const int grid = static_cast<int>(
+      std::max<int64_t>(1, std::min<int64_t>(want, static_cast<int64_t>(device_sm_count()) * 8)));
+  if (few)
+    lsq_warp_kernel<Q, SIGNED, G><<<grid, kLsqThreads, 0, stream>>>(w, ngroups, steps, step,
+                                                                    t.codes, t.scales, status);
+  else
+    lsq_kernel<Q, SIGNED, G><<<grid, kLsqThreads, 0, stream>>>(w, ngroups, steps, step, t.codes,
+                                                               t.scales, status);
+  return cudaGetLastError();
+}
+
 template <int Q, bool SIGNED>
 cudaError_t lsq_g(const float* w, const sss_qtensor_t& t, int steps, float step,
                   uint32_t* status, cudaStream_t stream) {
-  const int64_t ngroups = t.n * (t.k / t.group);
-  const int64_t want = (ngroups * (t.group / 32) + kLsqThreads - 1) / kLsqThreads;
-  const int grid = static_cast<int>(
-      std::max<int64_t>(1, std::min<int64_t>(want, static_cast<int64_t>(device_sm_count()) * 8)));
   switch (t.group) {
-    case 32:
-      lsq_kernel<Q, SIGNED, 32><<<grid, kLsqThreads, 0, stream>>>(w, ngroups, steps, step, t.codes,
-                                                                  t.scales, status);
-      break;
-    case 64:
-      lsq_kernel<Q, SIGNED, 64><<<grid, kLsqThreads, 0, stream>>>(w, ngroups, steps, step, t.codes,
-                                                                  t.scales, status);
-      break;
-    case 128:
-      lsq_kernel<Q, SIGNED, 128><<<grid, kLsqThreads, 0, stream>>>(w, ngroups, steps, step,
-                                                                   t.codes, t.scales, status);
-      break;
-    default:
-      return cudaErrorInvalidValue;
+    case 32: return lsq_run<Q, SIGNED, 32>(w, t, steps, step, status, stream);
+    case 64: return lsq_run<Q, SIGNED, 64>(w, t, steps, step, status, stream);
+    case 128: return lsq_run<Q, SIGNED, 128>(w, t, steps, step, status, stream);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
