@@ -13,6 +13,13 @@
 //    subtract and a multiply, and rounds to fp16.  A code field masked in
 //    place is the fp16 subnormal u 2^pos 2^-24, exact; the staged x carries
 //    2^-pos.  The symmetric offset enters as the accumulator's start value.
+//  * The tensor core lines products up by the operands' exponent fields, so the
+//    leading zeros of a subnormal cost the result low bits.  At q = 2 the fields
+//    are taken as high in the mantissa as they go, pos 6 and 8 (at pos 0 .. 4 the
+//    error against 64 bits was 2e-6 of the result, 1e-7 to 2e-7 now; the symmetric
+//    grids' weights are exact in fp16 there, so that gemv_batch.cu has 2e-7 to
+//    4e-6).  At q = 4, pos 0 and 4, it is 5e-7 against 2e-4; CUT shapes, which the
+//    general kernel computes to 2e-7 .. 3e-7, take pos 2 and 6.
 //  * ldmatrix hands quad t the t-th 32-bit word of a row's 16 bytes.  q = 4:
 //    the words of one sub-chunk.  q = 2: 16 bytes are two sub-chunks, and one
 //    shuffle and two byte permutes give every quad eight codes of each.
@@ -177,6 +184,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int NBC = SH::NBC, SEG = SH::SEG, P = SH::P, SB = SH::SB, BS = SH::BS;
   constexpr int HALF = 1 << (Q - 1);
   constexpr int CPR = P / 16;  // 16-byte chunks of a row in a step
+  constexpr float kScale = Q == 2 ? 0x1p-18f : (CUT ? 0x1p-22f : 0x1p-24f);  // of the mmas' results
   extern __shared__ __align__(128) unsigned char smem[];
   cg::cluster_group cluster = cg::this_cluster();
   const int S = static_cast<int>(cluster.num_blocks()), lgS = 31 - __clz(S);
@@ -354,18 +362,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t pr[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        // field e: pos 0, 4, then 0, 4 after a shift by 8 (q = 4), or pos 0, 2,
-        // 4 and 0 after a shift by 6
-        constexpr float kMul[2][4] = {{1.f, 0.0625f, 1.f, 0.0625f}, {1.f, 0.25f, 0.0625f, 1.f}};
+        // code e: pos 0, 4, then 0, 4 after a shift by 8 (q = 4; CUT: 2, 6, 2, 6, x
+        // with 2^(2 - pos)); codes 0, 3, then 2, 1 after a shift by 4: pos 8, 6, 8, 6
+        // (q = 2; x with 2^(6 - pos))
+        constexpr float kMul[2][4] = {{1.f, 0.0625f, 1.f, 0.0625f}, {0.25f, 1.f, 0.25f, 1.f}};
         const float mul = kMul[Q == 4 ? 0 : 1][e];
-        __half2 hv = __floats2half2_rn(f[e] * mul, f[e + 4] * mul);
+        const int c = Q == 2 && (e & 1) ? 4 - e : e;
+        __half2 hv = __floats2half2_rn(f[c] * mul, f[c + 4] * mul);
         pr[e] = *reinterpret_cast<uint32_t*>(&hv);
         // x as the operand holds it (exactly x from 2^-13 on): the row sum has to
         // meet the codes' product with the same values, or what fp16 rounded off
         // smaller ones would be left over times 2^(q-1)
         const float2 held = __half22float2(hv);
-        f[e] = held.x * (1.f / mul);
-        f[e + 4] = held.y * (1.f / mul);
+        f[c] = held.x * (1.f / mul);
+        f[c + 4] = held.y * (1.f / mul);
       }
       float sum = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
 #pragma unroll
@@ -375,10 +385,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(pr[0]), "r"(pr[1]),
                    "r"(pr[2]), "r"(pr[3])
                    : "memory");
-      // the row-sum term on the mma's scale 2^-24: times -2^(q-1) as the start
+      // the row-sum term on the mma's scale: times -2^(q-1) as the start
       // value of the symmetric grids, plain for the min
       if (lane % (G / 8) == 0)
-        b0[r] = ASYM ? sum * 0x1p-24f : -static_cast<float>(HALF) * 0x1p-24f * sum;
+        b0[r] = ASYM ? sum * kScale : -static_cast<float>(HALF) * kScale * sum;
     }
   };
   const int ul0 = warp & ((1 << lgu) - 1);
@@ -490,13 +500,17 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int h = 0; h < 4; ++h) {
             if constexpr (Q == 4) {
-              const uint32_t v = j ? w[0][h] >> 8 : w[0][h];
-              f0[h] = v & 0x000F000Fu;
-              f1[h] = v & 0x00F000F0u;
+              // pos 0 and 4; CUT: 2 and 6, for one more shift (see the top)
+              const uint32_t v = CUT ? (j ? w[0][h] >> 6 : w[0][h] << 2) : (j ? w[0][h] >> 8 : w[0][h]);
+              f0[h] = v & (CUT ? 0x003C003Cu : 0x000F000Fu);
+              f1[h] = v & (CUT ? 0x03C003C0u : 0x00F000F0u);
             } else {
               const uint32_t v = w[sc & 1][h];
-              f0[h] = v & (j ? 0x00300030u : 0x00030003u);
-              f1[h] = j ? (v >> 6) & 0x00030003u : v & 0x000C000Cu;
+              // both bytes of a half hold the same four codes: code 0 at pos 8, 3 at
+              // pos 6, and after a shift by 4 code 2 at pos 8, 1 at pos 6
+              const uint32_t vs = j ? v >> 4 : v;
+              f0[h] = vs & 0x03000300u;
+              f1[h] = vs & 0x00C000C0u;
             }
           }
 #pragma unroll
@@ -606,7 +620,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 4
         for (int w = 0; w < KW; ++w) sum += pb[w * share];
       }
-      sum *= 0x1p24f;
+      sum *= 1.f / kScale;
       if (__builtin_expect(!(fabsf(sum) <= 0x1.fffffep127f), 0))
         sum = plain_dot<Q, ASYM, G>(a, r, col);
       a.y[static_cast<int64_t>(col) * a.n + r] = sum;

@@ -96,7 +96,7 @@ def test_gemv_cluster_small_activations(mag, q, grid, k):
     # that of the rounded values, symmetric offset and minimum included
     qt = sss.sss_quantize(inputs.student_t_weights_cuda(100, k, 13, outliers=False), q, 32, grid)
     x = (inputs.normal_bf16_cuda((5, k), 14).float() * mag).bfloat16()
-    pos = torch.tensor([0., 4., 0., 4.] if q == 4 else [0., 2., 4., 0.], device="cuda")
+    pos = torch.tensor([0., 4., 0., 4.] if q == 4 else [2., 0., 2., 0.], device="cuda")
     p2 = torch.exp2(pos.repeat(k // 4))  # of elements e and e + 4 of every eight
     held = (x.float() / p2).half().double() * p2.double()
     w = sss.sss_dequantize(qt).double()
@@ -128,3 +128,17 @@ def test_gemv_cluster_activations_beyond_fp16(q, grid, n, k):
     for b in (7, 9, 15):  # +-inf by the weight's sign, NaN where it is zero
         assert torch.equal(y[b].isnan(), ref[b].isnan())
         assert torch.equal(y[b].nan_to_num(0.0), ref[b].float().nan_to_num(0.0))
+
+
+@pytest.mark.parametrize("batch", [3, 16])
+@pytest.mark.parametrize("n,k,g,grid", [
+    (200, 1024, 32, sss.GRID_SIGNED_SYM), (200, 1024, 128, sss.GRID_UNSIGNED_SYM),
+    (2048, 2048, 64, sss.GRID_SIGNED_SYM), (600, 1056, 32, sss.GRID_SIGNED_SYM),
+])
+def test_gemv_cluster_q2_symmetric_is_exact_products(n, k, g, grid, batch):
+    # fp32 sums of exact products: of the order of the square root of the chain's
+    # length, up to 64 additions here, times 2^-24
+    qt = sss.sss_quantize(inputs.student_t_weights_cuda(n, k, 17, outliers=False), 2, g, grid)
+    x = inputs.normal_bf16_cuda((batch, k), 18)
+    ref = x.double() @ sss.sss_dequantize(qt).double().T
+    assert ((sss.sss_gemv(qt, x) - ref).norm() / ref.norm()).item() <= 8 * 2.0**-24
