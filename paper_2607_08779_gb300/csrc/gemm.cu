@@ -34,9 +34,14 @@
 //              after a tile's last step the same warps drain its fp32
 //              accumulator with tcgen05.ld and store Y (for a fixed token, a
 //              warp writes 32 consecutive floats).
-// Tensor memory (512 columns): the fp32 accumulator (two for BN <= 128), then
-// four A stages of 64 columns (lane = row, two k-consecutive halves per 32-bit
-// column).
+// Tensor memory (512 columns): 256 columns of fp32 accumulators, then four A
+// stages of 64 columns (lane = row, two k-consecutive halves per 32-bit column).
+// Where every CTA has one item only (SOLO; up to 128 tokens per tile), its 256 / BN
+// accumulators each take a share of the steps and are added in fp32 at the end: the
+// tensor core's sums truncate, so the error grows with the length of the chain
+// (q = 2, whose weights are exact in fp16: 5120 x 5120 at 256 tokens 5.1e-6 -> 2.4e-6
+// against 64 bits, 4096 x 14336 at 17 3.5e-6 -> 7.7e-7).  With no further item to
+// run ahead to, the second accumulator would lie idle.
 // What bounds it: at BN = 256 the MMAs (1025 cycles a step; 512 per k-block is
 // the pipe's rate), 86 % of cuBLAS's burst rate at 2048 tokens with the
 // conversion of X (14336 x 4096 q = 4: 144 us; 192 us when a tile's k-blocks
@@ -212,18 +217,34 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
       : "memory");
 }
 
+// W = 16 or 32 consecutive columns, to be waited for
+template <int W>
+__device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[W]) {
+  if constexpr (W == 16) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+  } else {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+          "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
+          "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
+          "=r"(r[31])
+        : "r"(taddr));
+  }
+}
+
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-        "=r"(r[31])
-      : "r"(taddr));
+  tmem_ld_async<32>(taddr, r);
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
@@ -407,7 +428,7 @@ constexpr int kAStages = 4; // A operand steps (two k-blocks) in tensor memory
 
 // Shared memory: XS activation tiles (1024-aligned for the 128-byte
 // swizzle), then with CT the code tiles, then the barriers.
-template <int BN, int Q, bool CT>
+template <int BN, int Q, bool CT, bool SOLO>
 struct Smem {
   static constexpr int XS = BN == 256 ? 3 : 4;               // activation stages (steps)
   static constexpr int WS = BN == 256 ? 2 : 4;               // code tiles in flight
@@ -416,13 +437,14 @@ struct Smem {
   static constexpr int W_OFF = XS * 2 * X_BYTES;
   static constexpr int BAR_OFF = W_OFF + WS * W_BYTES;
   static constexpr bool JOINT = XS == kAStages;              // one stage for X and A
-  static constexpr int NB = BN == 256 ? 1 : 2;               // accumulators
+  static constexpr int NB = BN == 256 || SOLO ? 1 : 2;       // accumulators, item by item
+  static constexpr int PARTS = SOLO ? 256 / BN : 1;          // accumulators of an item
   static constexpr int NBAR = XS + 2 * kAStages + 2 * WS + 2 * NB + 1;
   static constexpr int TOTAL = BAR_OFF + NBAR * 8 + 16 + 1024;  // + align slack
-  static constexpr int A_COL = NB * BN;           // first A-stage column in tensor memory
+  static constexpr int A_COL = 256;               // first A-stage column in tensor memory
   static_assert(kAStages == 4 && WS % 2 == 0 && XS <= kAStages, "see kAStages");
   static_assert(TOTAL <= 227 * 1024, "shared memory per CTA");
-  static_assert(NB * BN + 64 * kAStages <= 512, "tensor memory holds accumulators and A stages");
+  static_assert(NB * PARTS * BN <= A_COL && A_COL + 64 * kAStages <= 512, "tensor memory");
 };
 constexpr int kTmemCols = 512;  // one CTA per SM
 
@@ -575,14 +597,16 @@ __device__ __forceinline__ bool sum_splits(const GemmArgs& a, const Item& e, int
 // MMAs run through the drain as well.  (One CTA per item spent about 9000 of
 // 27000 cycles at 128 tokens and k = 4096 on its start and end.)
 //
+// SOLO: no more items than CTAs; the loops over items then end with the first.
+//
 // CT: the packed codes arrive by TMA (rows of k q / 8 bytes, a multiple of
 // 16); otherwise (q = 3 with k an odd multiple of 64) each dequantising
 // thread loads its own from global memory one step ahead.
-template <int Q, bool ASYM, int BN, bool CT>
+template <int Q, bool ASYM, int BN, bool CT, bool SOLO>
 __global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmArgs a) {
-  using S = Smem<BN, Q, CT>;
-  constexpr int XS = S::XS, WS = S::WS, NB = S::NB;
+  using S = Smem<BN, Q, CT, SOLO>;
+  constexpr int XS = S::XS, WS = S::WS, NB = S::NB, PARTS = S::PARTS;
   extern __shared__ unsigned char smem_raw[];
   // 1024-byte alignment for the swizzle atoms
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -722,6 +746,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         near = (near << 1) & 15u;
       }
       P += (w.nsteps + 1) & ~1;
+      if constexpr (SOLO) break;
     }
     if (*abort) {
       // let this CTA's copies still in flight land before the CTA exits (of a
@@ -748,7 +773,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int it = blockIdx.x; it < a.items && go; it += gridDim.x, ++n) {
       const Item w = item_of(a, it, BN);
       const int buf = n % NB;
-      const uint32_t acc = tm + static_cast<uint32_t>(buf * BN);
+      uint32_t acc = tm + static_cast<uint32_t>(buf * BN);
+      const int share = (w.nsteps + PARTS - 1) / PARTS;  // steps per accumulator
+      int turn = P;                                      // the next one's first
       // the accumulator's previous item has been drained
       const bool fr = mbar_wait(&acc_free[buf], (static_cast<uint32_t>(n / NB) & 1u) ^ 1u, abort);
       if (!__all_sync(0xffffffffu, fr)) break;
@@ -775,12 +802,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             phx ^= 1u;
           }
           constexpr int kNext[4] = {1, 2, 3, 0};
+          const bool fresh = P0 + s == turn;
+          if (PARTS > 1 && fresh) {
+            acc += turn == P ? 0u : BN;
+            turn += share;
+          }
           const bool next = mbar_test_wait(&full_a[kNext[s]], (used >> kNext[s]) & 1u) &&
                             mbar_test_wait(&full_x[S::JOINT ? kNext[s] : sx],
                                            S::JOINT ? (used >> kNext[s]) & 1u : phx);
           if (elect_one()) {
             const uint32_t ta = tm + static_cast<uint32_t>(S::A_COL + 64 * s);
-            umma_kblock(acc, ta, bd, idesc, P0 + s == P ? 1u : 0u);
+            umma_kblock(acc, ta, bd, idesc, fresh ? 1u : 0u);
             if (2 * (P0 + s - P) + 1 < w.nkb) umma_kblock(acc, ta + 32, bd + bstep, idesc, 0u);
             umma_commit(&empty[s]);  // frees both operands' stages once these MMAs complete
           }
@@ -790,6 +822,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (elect_one()) umma_commit(&done[buf]);
       __syncwarp();
       P += (w.nsteps + 1) & ~1;
+      if constexpr (SOLO) break;
     }
     if (*abort) {  // MMAs still in flight must retire before the CTA's memory goes
       int drain = 0;
@@ -942,7 +975,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int pad = (w.nsteps + 1) & ~1;
       for (int p = ((slot - P) & 3) + (begun ? 4 : 0); p < pad && ok; p += 4) do_step(p, n == 0);
       begun = false;
-      if (ok && it + static_cast<int>(gridDim.x) < a.items) {
+      if (!SOLO && ok && it + static_cast<int>(gridDim.x) < a.items) {
         P += pad;
         start_item(it + gridDim.x);
         const int p = (slot - P) & 3;
@@ -975,9 +1008,39 @@ __global__ void __launch_bounds__(kThreads, 1)
           __syncwarp();
           if (lane == 0) mbar_arrive(&acc_free[buf]);
         };
-        if (32 * slot >= BN) release();
+        if constexpr (SOLO) {
+          // the groups take BN / 4 columns each, of all accumulators at once
+          constexpr int W = BN / 4;
+          const int c0 = W * slot;
+          const int share = (e.nsteps + PARTS - 1) / PARTS;
+          uint32_t v[PARTS][W];
+#pragma unroll
+          for (int p = 0; p < PARTS; ++p)
+            tmem_ld_async<W>(lane_base + static_cast<uint32_t>(p * BN + c0), v[p]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int p = 0; p < PARTS; ++p)
+#pragma unroll
+            for (int c = 0; c < W; ++c) asm volatile("" : "+r"(v[p][c]));  // (not before the wait)
+#pragma unroll
+          for (int p = 1; p < PARTS; ++p)
+            if (p * share < e.nsteps) {  // (the others were not written)
+#pragma unroll
+              for (int c = 0; c < W; ++c)
+                v[0][c] = __float_as_uint(__uint_as_float(v[0][c]) + __uint_as_float(v[p][c]));
+            }
+          if (erok) {
+            float* d = dst + c0 * ld;
+#pragma unroll
+            for (int c = 0; c < W; ++c) {
+              if (c0 + c < mleft) *d = __uint_as_float(v[0][c]);
+              d += ld;
+            }
+          }
+        }
+        if (!SOLO && 32 * slot >= BN) release();
 #pragma unroll 1
-        for (int c0 = 32 * slot; c0 < BN; c0 += 128) {
+        for (int c0 = 32 * slot; !SOLO && c0 < BN; c0 += 128) {
           uint32_t v[32];
           tmem_ld32(lane_base + static_cast<uint32_t>(buf * BN + c0), v);
           if (c0 + 128 >= BN) release();
@@ -994,6 +1057,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // (all 16 warps meet here for each item, so that one whose wait ran out
       // leaves no other at the barriers of the sum)
       if (split && !sum_splits(a, e, BN, ok, last)) ok = false;
+      if constexpr (SOLO) break;
     }
     if constexpr (!ASYM)
       big = __half2float(__hmax(__low2half(smax), __high2half(smax))) *
@@ -1168,9 +1232,9 @@ struct GemmCall {
   int* cnt;
 };
 
-template <int Q, bool ASYM, int BN, bool CT>
+template <int Q, bool ASYM, int BN, bool CT, bool SOLO>
 cudaError_t run_gemm(const GemmCall& c) {
-  using S = Smem<BN, Q, CT>;
+  using S = Smem<BN, Q, CT, SOLO>;
   const sss_qtensor_t& t0 = *c.ts[0];  // k, q, group and grid are those of every matrix
   EncodeTiledFn enc = tensor_map_encoder();
   if (enc == nullptr) return cudaErrorNotSupported;
@@ -1218,7 +1282,7 @@ cudaError_t run_gemm(const GemmCall& c) {
     a.job[j].tile0 = tile0;
     tile0 += (t.n + kBM - 1) / kBM;
   }
-  auto kern = gemm_kernel<Q, ASYM, BN, CT>;
+  auto kern = gemm_kernel<Q, ASYM, BN, CT, SOLO>;
   cudaError_t e = ensure_smem(kern, S::TOTAL);
   if (e != cudaSuccess) return e;
   a.njobs = c.count;
@@ -1259,10 +1323,12 @@ cudaError_t run_gemm(const GemmCall& c) {
 
 template <int Q, bool ASYM, bool CT>
 cudaError_t gemm_bn(const GemmCall& c) {
+  const int64_t items = row_tiles(c.ts, c.count) * ((c.m + c.plan.bn - 1) / c.plan.bn) * c.plan.nsplit;
+  const bool solo = items <= device_sm_count();
   switch (c.plan.bn) {
-    case 64: return run_gemm<Q, ASYM, 64, CT>(c);
-    case 128: return run_gemm<Q, ASYM, 128, CT>(c);
-    default: return run_gemm<Q, ASYM, 256, CT>(c);
+    case 64: return solo ? run_gemm<Q, ASYM, 64, CT, true>(c) : run_gemm<Q, ASYM, 64, CT, false>(c);
+    case 128: return solo ? run_gemm<Q, ASYM, 128, CT, true>(c) : run_gemm<Q, ASYM, 128, CT, false>(c);
+    default: return run_gemm<Q, ASYM, 256, CT, false>(c);
   }
 }
 
