@@ -796,9 +796,12 @@ cudaError_t launch_g(int g, ClusterArgs& a, cudaStream_t stream) {
 // q = 2 and 4, any k; launch_gemv_cluster may still return
 // cudaErrorNotSupported (a k whose staged x fits no cluster), without having
 // launched anything.  Scale rows of 2-byte alignment come by loads that a warp
-// waits for, a block at a time: with many groups of 32, few rows to share them
-// and little work per row, the general kernel is as fast or faster (300 x 2080,
-// q = 2, batch 2: 4.3 us against 4.9; 1024 x 4128: 5.0 against 4.8).
+// waits for, a block at a time: with groups of 32, long rows, few of them to share
+// the wait and little work per row, the general kernel is faster.  Time here over
+// there, the geometric mean over n = 32 .. 512 and k = 2080 .. 12320: at batch 2
+// 1.06 (q = 2 symmetric), 1.15 (q = 2 min-max), 0.97 (q = 4 symmetric) and 1.12
+// (q = 4 min-max), at batch 4 0.95, 1.02, 0.92 and 1.01; k = 1056 and 1568 0.73 to
+// 1.00.  The error here is a sixth of the general kernel's, so a tie comes here.
 bool gemv_cluster_eligible(const sss_qtensor_t& t, const uint16_t* x, int batch, const float* y) {
   auto al = [](const void* p, size_t b) { return (reinterpret_cast<uintptr_t>(p) % b) == 0; };
   if (t.q == 3 || batch < 2 || batch > 16) return false;
@@ -806,7 +809,9 @@ bool gemv_cluster_eligible(const sss_qtensor_t& t, const uint16_t* x, int batch,
   if (t.n > (int64_t{1} << 30)) return false;
   if (!al(t.codes, 16) || !al(t.scales, 2) || !al(x, 16) || !al(y, 4)) return false;
   if (t.grid == SSS_GRID_ASYM && !al(t.mins, 2)) return false;
-  if (t.group == 32 && t.k / 32 % 2 != 0 && batch <= 4 && t.n <= 512 && t.k >= 1024) return false;
+  if (t.group == 32 && t.k / 32 % 2 != 0 && batch == 2 && t.n <= 512 && t.k >= 2048 &&
+      (t.q == 2 || t.grid == SSS_GRID_ASYM))
+    return false;
   return true;
 }
 
