@@ -146,21 +146,27 @@ sss_status_t sss_dequantize(const sss_qtensor_t* qt, void* out,
  * sss_gemv -- decode GEMV y[b][r] = sum_k w^[r][k] * x[b][k] with the
  * dequantisation fused (Appendix B.3: y = sum_b s * (integer dot) for the
  * symmetric formats, plus the row-sum term sum_b m * sum_{k in b} x for
- * ASYM).  fp32 accumulation; deterministic (no atomics).  At batch 1, and at
- * batch 2..16 for q = 2 and 4, the integer codes meet the activations exactly
- * and the group scale is applied in fp32; so too for q = 3 with k not a multiple
- * of 256.  (At batch 2..16 an activation enters as fp16 x * 2^-p, p = 0, 2 or 4
- * the bit offset of the code's field: exactly x for 2^-13 <= |x| <= 65504, below
- * that within 2^-21 of it.  For q = 2 and 4 the outputs of a batch row with larger
- * or infinite activations are computed by plain fp32 products of w^ and x, many
- * times slower; for q = 3 they are infinite or NaN.)  Otherwise, for q = 3, the
- * batch fills the tensor-core columns across groups, so each weight enters the
- * product as w^ rounded once to fp16 (<= 2^-11 relative, as in sss_gemm), times
- * 2^p (p = 0, 2 or 4, the bit offset of the code's field).  That operand fits
- * fp16 while |w^| * 2^p < 65520; at batch 2..16 with k a multiple of 256,
- * whatever q, every group whose scale could break this raises SSS_FLAG_RANGE
- * (checked per scale, conservatively: |s| * 2^(q-1) * 16 >= 65520 for the
- * symmetric grids, (|s| * (2^q - 1) + |m|) * 16 >= 65520 for ASYM).
+ * ASYM).  fp32 accumulation; deterministic (no atomics).
+ * At batch 1 the integer codes meet the activations exactly and the group scale is
+ * applied in fp32.  So it is at batch 2..16 for q = 2 and 4, and whenever k is not a
+ * multiple of 256, with these limits:
+ *   - an activation enters as fp16 x * 2^-p, p = 0, 2 or 4: exactly x for 2^-13 <=
+ *     |x| <= 65504.  Smaller ones are rounded, to within 2^-21.  With larger or
+ *     infinite ones, the outputs of their batch row are computed by plain fp32
+ *     products of w^ and x, many times slower (q = 2 and 4, k a multiple of 256), or
+ *     may be infinite or NaN (else);
+ *   - the staged activations fit the shared memory: at batch 2..8, k up to 30720 at
+ *     least (q = 4 ASYM, group 32; 38912 and more for the others); at batch 9..16
+ *     k <= 12288 for q = 4 ASYM (17920 with group 128), 16384, 17920 or 21504 for q
+ *     = 4 symmetric and 22528, 24576 or 28672 for q = 2 (group 32, 64 or 128).
+ * Otherwise (k a multiple of 256 and q = 3 or a longer k) the batch fills the
+ * tensor-core columns across groups, so each weight enters the product as w^
+ * rounded once to fp16 (<= 2^-11 relative, as in sss_gemm), times 2^p (p = 0, 2 or
+ * 4, the bit offset of the code's field).  That operand fits fp16 while |w^| * 2^p <
+ * 65520; at batch 2..16 with k a multiple of 256, whatever q, every group whose
+ * scale could break this raises SSS_FLAG_RANGE (checked per scale, conservatively:
+ * |s| * 2^(q-1) * 16 >= 65520 for the symmetric grids, (|s| * (2^q - 1) + |m|) * 16
+ * >= 65520 for ASYM).
  *   qt        [in]  packed tensor; codes 16-byte aligned, scales/mins 4-byte
  *                   aligned.
  *   x_bf16    [in]  device bf16 [batch][k], 16-byte aligned.

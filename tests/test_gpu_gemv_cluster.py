@@ -142,3 +142,23 @@ def test_gemv_cluster_q2_symmetric_is_exact_products(n, k, g, grid, batch):
     x = inputs.normal_bf16_cuda((batch, k), 18)
     ref = x.double() @ sss.sss_dequantize(qt).double().T
     assert ((sss.sss_gemv(qt, x) - ref).norm() / ref.norm()).item() <= 8 * 2.0**-24
+
+
+@pytest.mark.parametrize("q,grid,g,batch,k", [
+    (4, sss.GRID_ASYM, 32, 16, 12288), (4, sss.GRID_ASYM, 64, 9, 12288),
+    (4, sss.GRID_SIGNED_SYM, 32, 16, 16384), (4, sss.GRID_SIGNED_SYM, 128, 9, 21504),
+    (2, sss.GRID_ASYM, 32, 16, 22528), (2, sss.GRID_SIGNED_SYM, 128, 9, 28672),
+    (4, sss.GRID_ASYM, 32, 8, 30720), (4, sss.GRID_SIGNED_SYM, 64, 2, 45056),
+])
+def test_gemv_cluster_longest_rows(q, grid, g, batch, k):
+    # the longest k whose staged activations fit a cluster: fp32 sums; and the next
+    # multiple of 256, the batched kernel: weights rounded to fp16
+    for kk, tol in ((k, TOL), (k + 256, 2.0**-11)):
+        qt = sss.sss_quantize(inputs.student_t_weights_cuda(40, kk, 19, outliers=False), q, g, grid)
+        x = inputs.normal_bf16_cuda((batch, kk), 20)
+        y = sss.sss_gemv(qt, x)
+        ref = x.double() @ sss.sss_dequantize(qt).double().T
+        err = ((y - ref).abs().amax(1) / ref.abs().amax(1)).max().item()
+        assert err <= tol
+        if tol != TOL and q == 4:  # (symmetric weights at q = 2 are exact in fp16)
+            assert err > TOL
