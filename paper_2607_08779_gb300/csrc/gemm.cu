@@ -1175,39 +1175,62 @@ size_t split_bytes(int64_t rt, int64_t m, const GemmPlan& p) {
   return round256(static_cast<size_t>(p.nsplit) * m * rt * kBM * 4) + round256(tiles * 4);
 }
 
-// The plan of least estimated time, in SM cycles: each SM's share of the items,
-// an item at a time, plus the launch's start and end, and for K splits the last
-// arrival's sum of the partial tiles.  Per k-block 64- and 128-token tiles count
-// about 290 cycles (325-375 in a long loop) and 256-token tiles 512 (the
-// MMAs').  Splits end on code-tile boundaries and keep at least 8 k-blocks.
+// The plan: for each tile width the K split of least estimated SM cycles (the
+// k-blocks of a CTA, its start and end, and the last arrival's sum of the partial
+// tiles), then the width of least estimated time in ns (the rounds of items that the
+// busiest SM takes, what all items draw together, and a split's cost).  The second
+// estimate is fitted to 585 calls at q = 4 (n = 1024 .. 28672, k = 1024 .. 14336, m =
+// 17 .. 2048) at every width: off by 3, 5 and 7 % (64, 128 and 256 tokens); the
+// width chosen is within 0.2 % of the best one's time in the geometric mean.  (The
+// first estimate alone, 290 cycles per k-block for 64 and 128 tokens and 512 for
+// 256, took 128-token tiles too often: 14336 x 1024 at 256 tokens 15.6 us against
+// 13.1, 20000 x 1024 at 2048 93 against 75.)  Splits end on code-tile boundaries,
+// keep at least 8 k-blocks and only fill SMs that the tiles leave idle.
 // rt: the row tiles of all the call's matrices; ws: the bytes the partial tiles
-// must fit in.  K is split only to fill SMs that the tiles leave idle.
+// must fit in.
 GemmPlan plan_gemm(int64_t rt, int64_t k, int64_t m, size_t ws) {
+  struct Width {
+    int bn;
+    int64_t cycles, drain;  // per k-block, per item
+    int64_t start, item, kblock, load, split;  // ns
+  };
+  constexpr Width kWidths[] = {{64, 288, 600, 0, 1100, 153, 20, 2100},
+                               {128, 296, 600, 40, 1830, 138, 49, 2500},
+                               {256, 512, 2500, 170, 3200, 199, 97, 3200}};
   const int64_t sms = device_sm_count();
   const int64_t nkb = k / kBK;
   GemmPlan best{128, 1, static_cast<int>((nkb + kWK - 1) / kWK * kWK)};
-  int64_t best_cost = INT64_MAX;
-  for (int bn : {64, 128, 256}) {
-    if (bn > 64 && m <= bn / 2) break;
-    const int64_t per = bn == 256 ? 512 : 280 + bn / 8;
-    const int64_t tiles = rt * ((m + bn - 1) / bn);
+  int64_t best_ns = INT64_MAX;
+  for (const Width& w : kWidths) {
+    if (w.bn > 64 && m <= w.bn / 2) break;
+    const int64_t tiles = rt * ((m + w.bn - 1) / w.bn);
+    GemmPlan plan = best;
+    int64_t best_cycles = INT64_MAX;
     for (int64_t split = 1; split <= 32; ++split) {
       const int64_t chunk = ((nkb + split - 1) / split + kWK - 1) / kWK * kWK;
       if (split > 1 &&
           (chunk < 8 || (nkb + chunk - 1) / chunk != split || tiles * split > sms))
         continue;
-      const GemmPlan p{bn, static_cast<int>(split), static_cast<int>(chunk)};
+      const GemmPlan p{w.bn, static_cast<int>(split), static_cast<int>(chunk)};
       if (split > 1 &&
           (x16_bytes(m, k) > ws || x16_bytes(m, k) + split_bytes(rt, m, p) > ws))
         continue;
       const int64_t rounds = (tiles * split + sms - 1) / sms;
-      const int64_t drain = bn == 256 ? 2500 : 600;
       const int64_t sum = split > 1 ? 500 + split * m * rt * kBM * 4 / 1000 : 0;
-      const int64_t cost = rounds * (std::min(chunk, nkb) * per + drain) + 16 * bn + sum;
-      if (cost < best_cost) {
-        best_cost = cost;
-        best = p;
+      const int64_t cycles = rounds * (std::min(chunk, nkb) * w.cycles + w.drain) + sum;
+      if (cycles < best_cycles) {
+        best_cycles = cycles;
+        plan = p;
       }
+    }
+    const int64_t items = tiles * plan.nsplit, kbs = std::min<int64_t>(plan.chunk, nkb);
+    const int64_t rounds = (items + sms - 1) / sms;
+    const int64_t sum = plan.nsplit > 1 ? w.split + 6 * plan.nsplit * std::min<int64_t>(m, w.bn) : 0;
+    const int64_t ns =
+        w.start + rounds * (kbs * w.kblock + w.item) + items * kbs * w.load / sms + sum;
+    if (ns < best_ns) {
+      best_ns = ns;
+      best = plan;
     }
   }
   return best;
