@@ -43,8 +43,8 @@
 // against 64 bits, 4096 x 14336 at 17 3.5e-6 -> 7.7e-7).  With no further item to
 // run ahead to, the second accumulator would lie idle.
 // What bounds it: at BN = 256 the MMAs (1025 cycles a step; 512 per k-block is
-// the pipe's rate), 86 % of cuBLAS's burst rate at 2048 tokens with the
-// conversion of X (14336 x 4096 q = 4: 144 us; 192 us when a tile's k-blocks
+// the pipe's rate), 88 % of cuBLAS's burst rate at 2048 tokens with the
+// conversion of X (14336 x 4096 q = 4: 140 us; 192 us when a tile's k-blocks
 // each brought their own narrow code and scale tiles); at BN <= 128 the TMA
 // unit's rows and the way from L2 to the SM (650-750 cycles a step; the MMAs
 // need 512 at BN = 128); at few tokens the launch itself.

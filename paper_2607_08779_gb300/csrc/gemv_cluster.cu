@@ -37,12 +37,14 @@
 //    4096, took as long as a small matrix's weights); each warp stores its
 //    partial sums into the shared memory of the CTA that owns the outputs, and
 //    after one cluster barrier the owners add them in a fixed order.
-// Measured (q = 4, g = 32, batch 4 / 16): 14336 x 4096 11.4 / 15.8 us, 4096 x
-// 4096 5.3 / 8.8 us, 4096 x 14336 10.6 / 19.0 us; the kernel with the scaled
+// Measured (q = 4, g = 32, batch 4 / 16): 14336 x 4096 11.4 / 15.5 us, 4096 x
+// 4096 5.2 / 8.5 us, 4096 x 14336 10.5 / 18.7 us; the kernel with the scaled
 // fp16 operand took 13.3 / 18.1, 7.4 / 10.5 and 16.4 / 32.8 us.  Bound at batch
 // 4 by the start (launch, staging x: about 3500 cycles) and the copies in
 // flight, at batch 16 by instruction issue (about 450 instructions per step,
-// 45 % of the slots used).
+// 43 % of the slots used) and the mma chains behind it.  The min-max grid with
+// groups of 32 pays for its exactness at large n and k: 8192 x 16384 at batch 2
+// 28.6 us against 26.0 with fp16-rounded weights (q = 4).
 #include <cooperative_groups.h>
 #include <stdint.h>
 #include <string.h>

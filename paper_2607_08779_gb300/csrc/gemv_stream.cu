@@ -120,10 +120,10 @@ __device__ __forceinline__ uint32_t field_pair(const uint32_t* w, const uint32_t
 // keeps every element exact in fp16 whatever the activations' magnitude.
 // sbf[i] = {b_i, f_i}: f_i = 2^(24 - E_i) undoes both scalings in the
 // epilogue, and b_i is the row-sum term of Appendix B.3 on the mma's scale:
-// sum(x) * 2^(E_i - 24), times -2^(q-1) for the symmetric grids.  Four
-// threads share a sub-chunk (8 elements each: at k = 4096 every thread of the
-// CTA has one part); threads tid = 0 .. nthreads-1 (whole warps) share the
-// work; the caller synchronises.
+// sum(x) * 2^(E_i - 24), times -2^(q-1) for the symmetric grids.  Two
+// threads share a sub-chunk (16 elements each; four with 8 each took 1 to 3 %
+// longer over a decode step); threads tid = 0 .. nthreads-1 (whole warps) share
+// the work; the caller synchronises.
 //
 // With act_q8 the activations are first quantized to Q8_0 (act_q8.cuh; a
 // sub-chunk is one Q8_0 block): the staged operand is the int8 code q

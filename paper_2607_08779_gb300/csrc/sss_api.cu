@@ -201,7 +201,8 @@ sss_status_t sss_gemv(const sss_qtensor_t* qt, const uint16_t* x_bf16, int32_t b
   // and 4 (a Llama3-8B layer's seven matrices, q = 4 at batch 4: 54 us against
   // 70 us), the batched kernel (fp16 weight operand) for q = 3 and a k whose
   // staged x fits no cluster; shapes none takes (batch 1 and q = 3 with k not a
-  // multiple of 256, unaligned buffers): the general kernel
+  // multiple of 256, unaligned buffers, a few that gemv_cluster_eligible names):
+  // the general kernel
   if (batch == 1 && gemv_stream_eligible(*qt, x_bf16)) {
     const sss_qtensor_t* one[1] = {qt};
     float* yy[1] = {y};

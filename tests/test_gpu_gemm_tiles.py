@@ -29,8 +29,8 @@ def test_gemm_several_tiles_per_cta(q, g, k, grid, m):
 
 
 @pytest.mark.parametrize("n,k,m,chain", [
-    (1024, 1152, 256, 5 * 8),     # 9 steps of 8 MMAs over the four accumulators of a 64-token tile, K split in two
-    (4096, 14336, 512, 56 * 8),   # 112 steps over the two of a 128-token tile
+    (1024, 1152, 256, 5 * 8),     # 9 steps of 8 MMAs over the four accumulators of a 64-token tile, or two
+    (4096, 14336, 512, 56 * 8),   # 112 steps: K split in two, or the two of a 128-token tile
     (512, 4096, 40, 8 * 8),
 ])
 def test_gemm_chains_of_accumulation_are_divided(n, k, m, chain):
